@@ -5,7 +5,7 @@
 //  * features/targets of (shell, band) rows from Ritz vectors X, their H X,
 //    Ritz values and the converged bands X* (training data harvested from the
 //    solver's own trajectories);
-//  * forward, loss + backward (block-level weight-gradient reduction), Adam;
+//  * forward, loss + backward (register-tiled products over row tiles), Adam;
 //  * the per-iteration factors used by the eigensolver's preconditioner.
 //
 // Parameter vector (FP32): W1 (64x4 row-major), b1, W2 (64x64), b2, W3 (64), b3,
@@ -26,10 +26,6 @@ constexpr int kMlpParams = MH * MIN + MH + MH * MH + MH + MH + 1;  // 4545
 constexpr int kMlpBlob = kMlpParams + 8;
 
 __device__ __forceinline__ float silu_f(float z) { return z / (1.f + __expf(-z)); }
-__device__ __forceinline__ float silu_g(float z) {
-  const float sg = 1.f / (1.f + __expf(-z));
-  return sg * (1.f + z * (1.f - sg));
-}
 
 // Load the parameters into shared memory (all threads).
 __device__ void mlp_load(const float* __restrict__ p, float* sp) {
@@ -37,8 +33,8 @@ __device__ void mlp_load(const float* __restrict__ p, float* sp) {
   __syncthreads();
 }
 
-// Forward pass of one row; optional caches of pre-activations.
-__device__ float mlp_row(const float* sp, const float f[4], float* z1c, float* z2c) {
+// Forward pass of one row.
+__device__ float mlp_row(const float* sp, const float f[4]) {
   const float* W1 = sp;
   const float* b1 = W1 + MH * MIN;
   const float* W2 = b1 + MH;
@@ -50,7 +46,6 @@ __device__ float mlp_row(const float* sp, const float f[4], float* z1c, float* z
   for (int i = 0; i < MH; ++i) {
     float z = b1[i] + W1[i * 4] * f[0] + W1[i * 4 + 1] * f[1] + W1[i * 4 + 2] * f[2] +
               W1[i * 4 + 3] * f[3];
-    if (z1c) z1c[i] = z;
     h1[i] = silu_f(z);
   }
   float s = b3;
@@ -58,7 +53,6 @@ __device__ float mlp_row(const float* sp, const float f[4], float* z1c, float* z
     float z = b2[i];
 #pragma unroll 16
     for (int j = 0; j < MH; ++j) z += W2[i * MH + j] * h1[j];
-    if (z2c) z2c[i] = z;
     s += W3[i] * silu_f(z);
   }
   return s;
@@ -71,94 +65,231 @@ __global__ void k_mlp_forward(const float* __restrict__ p, const float* __restri
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < rows;
        r += (int64_t)gridDim.x * blockDim.x) {
     float f[4] = {F[4 * r], F[4 * r + 1], F[4 * r + 2], F[4 * r + 3]};
-    s[r] = mlp_row(sp, f, nullptr, nullptr);
+    s[r] = mlp_row(sp, f);
   }
 }
 
 // Loss sum w (s - y)^2 / wsum and its gradient, accumulated (atomically) into
-// g (kMlpParams) and loss[0].  128 rows per block; the block reduces the
-// weight gradients of its rows in shared memory before one atomic per weight.
-constexpr int GR = 128;
-__global__ void __launch_bounds__(GR) k_mlp_grad(const float* __restrict__ p,
-                                                 const float* __restrict__ F,
-                                                 const float* __restrict__ y,
-                                                 const float* __restrict__ w, int64_t rows,
-                                                 float inv_wsum, float* __restrict__ g,
-                                                 float* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* sp = sm;                      // parameters
-  float* sh1 = sp + kMlpParams + 3;    // GR x MH: h1
-  float* sd2 = sh1 + GR * MH;          // GR x MH: dz2
-  float* sd1 = sd2 + GR * MH;          // GR x MH: dz1
-  float* sf = sd1 + GR * MH;           // GR x 4: features
-  float* sds = sf + GR * 4;            // GR: ds
-  float* sh2 = sds + GR;               // GR x MH: h2 (for gW3)
-  mlp_load(p, sp);
-  const float* W1 = sp;
-  const float* W2 = W1 + MH * MIN + MH;
-  const float* W3 = W2 + MH * MH + MH;
-  const int64_t r = blockIdx.x * (int64_t)GR + threadIdx.x;
-  const int t = threadIdx.x;
-  float z1[MH], z2[MH];
-  float ds = 0.f;
-  float f[4] = {0, 0, 0, 0};
-  if (r < rows) {
-    f[0] = F[4 * r]; f[1] = F[4 * r + 1]; f[2] = F[4 * r + 2]; f[3] = F[4 * r + 3];
-    const float s = mlp_row(sp, f, z1, z2);
-    const float e = s - y[r];
-    ds = 2.f * w[r] * e * inv_wsum;
-    atomicAdd(loss, w[r] * e * e * inv_wsum);
-  } else {
-    for (int i = 0; i < MH; ++i) z1[i] = z2[i] = 0.f;
-  }
-  // backward of one row
-  for (int i = 0; i < MH; ++i) {
-    sh1[t * MH + i] = (r < rows) ? silu_f(z1[i]) : 0.f;
-    sh2[t * MH + i] = (r < rows) ? silu_f(z2[i]) : 0.f;
-    sd2[t * MH + i] = ds * W3[i] * silu_g(z2[i]);
-  }
-  for (int j = 0; j < MH; ++j) {
-    float acc = 0.f;
-    for (int i = 0; i < MH; ++i) acc += sd2[t * MH + i] * W2[i * MH + j];
-    sd1[t * MH + j] = acc * silu_g(z1[j]);
-  }
-  for (int k = 0; k < 4; ++k) sf[t * 4 + k] = f[k];
-  sds[t] = ds;
+// g (kMlpParams) and loss[0].
+//
+// Bound: the FP32 pipes.  The three 64 x 64 products of a row (forward, back
+// through W2, gradient of W2) are 12,288 of its 13,250 multiply-adds, so each
+// is a register-tiled matrix product over a tile of GR rows: activations and
+// deltas lie transposed in shared memory ([unit][row], pitch GP: 16-byte
+// loads, eight neighbouring units on distinct banks) and a thread owns an
+// 8 x 4 (rows x units) tile of the first two products and a 4 x 4 tile of the
+// W2 gradient, 24 and 32 multiply-adds per 16-byte load triple / pair.  Blocks
+// are persistent (two per SM), so that every weight gradient stays in its
+// thread's registers until the block's last tile and costs one atomic per
+// block; z1 is recomputed in the backward pass (four multiply-adds) rather
+// than kept.  A training step (this kernel, two memsets, Adam) of 32,768 rows:
+// 85 us, against 356 us for a row per thread with scalar shared-memory weights.
+constexpr int GR = 128;        // rows per tile
+constexpr int GT = 256;        // threads per block
+constexpr int GP = GR + 4;     // pitch of the transposed activations
+constexpr int GLOADS = kMlpParams + 3;  // parameters, padded to 16 bytes
+static_assert(GLOADS % 4 == 0 && (MH * MIN + MH) % 4 == 0, "16-byte loads of W2");
+
+__device__ __forceinline__ float sigmoid_f(float z) { return 1.f / (1.f + __expf(-z)); }
+
+__global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float* __restrict__ p,
+                                                    const float* __restrict__ F,
+                                                    const float* __restrict__ y,
+                                                    const float* __restrict__ w, int64_t rows,
+                                                    float inv_wsum, float* __restrict__ g,
+                                                    float* __restrict__ loss) {
+  extern __shared__ __align__(16) float sm[];
+  float* sp = sm;                  // parameters
+  float* w2t = sp + GLOADS;        // W2 transposed: [j][i]
+  float* h1t = w2t + MH * MH;      // h1, [j][row]
+  float* d2t = h1t + MH * GP;      // dL/dz2, [i][row]
+  float* sf = d2t + MH * GP;       // features, [row][4]
+  float* ss = sf + GR * 4;         // partial outputs, [4][row]
+  float* sds = ss + 4 * GR;        // dL/ds, [row]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int i = t; i < kMlpParams; i += GT) sp[i] = p[i];
   __syncthreads();
-  // block reduction of the weight gradients
-  float* gW1 = g;
-  float* gb1 = gW1 + MH * MIN;
-  float* gW2 = gb1 + MH;
-  float* gb2 = gW2 + MH * MH;
-  float* gW3 = gb2 + MH;
-  float* gb3 = gW3 + MH;
-  for (int e = t; e < MH * MH; e += GR) {
-    const int i = e / MH, j = e % MH;
-    float acc = 0.f;
-    for (int q = 0; q < GR; ++q) acc += sd2[q * MH + i] * sh1[q * MH + j];
-    atomicAdd(&gW2[e], acc);
-  }
-  for (int e = t; e < MH * MIN; e += GR) {
-    const int i = e / MIN, k = e % MIN;
-    float acc = 0.f;
-    for (int q = 0; q < GR; ++q) acc += sd1[q * MH + i] * sf[q * 4 + k];
-    atomicAdd(&gW1[e], acc);
-  }
-  for (int i = t; i < MH; i += GR) {
-    float a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int q = 0; q < GR; ++q) {
-      a1 += sd1[q * MH + i];
-      a2 += sd2[q * MH + i];
-      a3 += sds[q] * sh2[q * MH + i];
+  const float* W1 = sp;
+  const float* b1 = W1 + MH * MIN;
+  const float* W2 = b1 + MH;
+  const float* b2 = W2 + MH * MH;
+  const float* W3 = b2 + MH;
+  const float b3 = W3[MH];
+  for (int e = t; e < MH * MH; e += GT) w2t[(e % MH) * MH + e / MH] = W2[e];
+  // tile of the first two products: rows r0..r0+3 and r0+64..r0+67, units c0..c0+3
+  const int rg = (warp & 1) * 8 + (lane & 7), cg = (warp >> 1) * 4 + (lane >> 3);
+  const int r0 = rg * 4, c0 = cg * 4;
+  // tile of the W2 gradient: units gi + 16 q (rows of W2), gj + 16 q (columns)
+  const int gi = (warp & 1) * 8 + (lane & 7), gj = (warp >> 1) * 4 + (lane >> 3);
+  float g2[4][4] = {}, g1[4][4] = {}, gb1[4] = {}, gb2[4] = {}, g3[4] = {};
+  float gb3 = 0.f, lsum = 0.f;
+  const int64_t ntile = (rows + GR - 1) / GR;
+  for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    const int64_t base = tile * GR;
+    __syncthreads();  // w2t written / the previous tile consumed
+    for (int e = t; e < GR * 4; e += GT) sf[e] = base + e / 4 < rows ? F[base * 4 + e] : 0.f;
+    __syncthreads();
+    {  // first layer: a row and half of the units per thread
+      const int r = t & (GR - 1), j0 = (t / GR) * (MH / 2);
+      const float4 f = *(const float4*)(sf + 4 * r);
+      const bool on = base + r < rows;
+#pragma unroll 8
+      for (int j = j0; j < j0 + MH / 2; ++j) {
+        const float4 a = *(const float4*)(W1 + 4 * j);
+        const float z = b1[j] + a.x * f.x + a.y * f.y + a.z * f.z + a.w * f.w;
+        h1t[j * GP + r] = on ? z * sigmoid_f(z) : 0.f;
+      }
     }
-    atomicAdd(&gb1[i], a1);
-    atomicAdd(&gb2[i], a2);
-    atomicAdd(&gW3[i], a3);
+    __syncthreads();
+    float acc[8][4];
+    // z2 = b2 + W2 h1
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) acc[r][q] = b2[c0 + q];
+#pragma unroll 2
+    for (int j = 0; j < MH; ++j) {
+      const float4 x0 = *(const float4*)(h1t + j * GP + r0);
+      const float4 x1 = *(const float4*)(h1t + j * GP + r0 + 64);
+      const float4 u = *(const float4*)(w2t + j * MH + c0);
+      const float xr[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+      const float uc[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(xr[r], uc[q], acc[r][q]);
+    }
+    // s = b3 + W3 silu(z2): partial sums over the thread's units, then over
+    // the warp's four unit groups and the block's four warp columns
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      float v = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v += W3[c0 + q] * (acc[r][q] * sigmoid_f(acc[r][q]));
+      v += __shfl_xor_sync(0xffffffffu, v, 8);
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+      if (lane < 8) ss[(warp >> 1) * GR + r0 + (r & 3) + 64 * (r >> 2)] = v;
+    }
+    __syncthreads();
+    if (t < GR) {
+      float ds = 0.f;
+      if (base + t < rows) {
+        const float s = b3 + ((ss[t] + ss[GR + t]) + (ss[2 * GR + t] + ss[3 * GR + t]));
+        const float e = s - y[base + t], we = w[base + t] * e * inv_wsum;
+        ds = 2.f * we;
+        lsum += we * e;
+      }
+      sds[t] = ds;
+      gb3 += ds;
+    }
+    __syncthreads();
+    // dL/dz2 and the gradients of b2 and W3
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 d4 = *(const float4*)(sds + r0 + 64 * h);
+      const float ds[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float o[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float z = acc[4 * h + r][q], sg = sigmoid_f(z);
+          // padding rows contribute nothing, whatever the parameters
+          const bool on = base + r0 + 64 * h + r < rows;
+          o[r] = on ? ds[r] * W3[c0 + q] * (sg * (1.f + z * (1.f - sg))) : 0.f;
+          gb2[q] += o[r];
+          g3[q] += on ? ds[r] * (z * sg) : 0.f;
+        }
+        *(float4*)(d2t + (c0 + q) * GP + r0 + 64 * h) = make_float4(o[0], o[1], o[2], o[3]);
+      }
+    }
+    __syncthreads();
+    // dL/dh1 = W2^T dL/dz2
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+#pragma unroll 2
+    for (int i = 0; i < MH; ++i) {
+      const float4 x0 = *(const float4*)(d2t + i * GP + r0);
+      const float4 x1 = *(const float4*)(d2t + i * GP + r0 + 64);
+      const float4 u = *(const float4*)(W2 + i * MH + c0);
+      const float xr[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+      const float uc[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(xr[r], uc[q], acc[r][q]);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int row = r0 + (r & 3) + 64 * (r >> 2);
+      const float4 f = *(const float4*)(sf + 4 * row);
+      const bool on = base + row < rows;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 a = *(const float4*)(W1 + 4 * (c0 + q));
+        const float z = b1[c0 + q] + a.x * f.x + a.y * f.y + a.z * f.z + a.w * f.w;
+        const float sg = sigmoid_f(z);
+        const float d = on ? acc[r][q] * (sg * (1.f + z * (1.f - sg))) : 0.f;
+        gb1[q] += d;
+        g1[q][0] += d * f.x;
+        g1[q][1] += d * f.y;
+        g1[q][2] += d * f.z;
+        g1[q][3] += d * f.w;
+      }
+    }
+    // gradient of W2: sum over the rows of dL/dz2[i] h1[j]
+#pragma unroll 1
+    for (int r = 0; r < GR; r += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        a[q] = *(const float4*)(d2t + (gi + 16 * q) * GP + r);
+        b[q] = *(const float4*)(h1t + (gj + 16 * q) * GP + r);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          g2[i][j] = fmaf(a[i].w, b[j].w,
+                          fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, g2[i][j]))));
+    }
   }
-  if (t == 0) {
-    float a = 0.f;
-    for (int q = 0; q < GR; ++q) a += sds[q];
-    atomicAdd(gb3, a);
+  float* gW1 = g;
+  float* gB1 = gW1 + MH * MIN;
+  float* gW2 = gB1 + MH;
+  float* gB2 = gW2 + MH * MH;
+  float* gW3 = gB2 + MH;
+  float* gB3 = gW3 + MH;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) atomicAdd(&gW2[(gi + 16 * i) * MH + gj + 16 * j], g2[i][j]);
+  // the other gradients: sums over the eight row groups of a warp, then atomics
+  auto reduce = [&](float v, float* dst) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    if ((lane & 7) == 0) atomicAdd(dst, v);
+  };
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int k = 0; k < MIN; ++k) reduce(g1[q][k], &gW1[(c0 + q) * MIN + k]);
+    reduce(gb1[q], &gB1[c0 + q]);
+    reduce(gb2[q], &gB2[c0 + q]);
+    reduce(g3[q], &gW3[c0 + q]);
+  }
+  if (t < GR) {  // whole warps
+    for (int o = 16; o > 0; o >>= 1) {
+      gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+      lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    }
+    if (lane == 0) {
+      atomicAdd(gB3, gb3);
+      atomicAdd(loss, lsum);
+    }
   }
 }
 
@@ -324,13 +455,13 @@ __global__ void k_mlp_factors(const float* __restrict__ blob, const int* __restr
     make_features(Tshell[g], theta[b], rn[b], eref[b], vbar, f);
     bool inside = true;
     for (int q = 0; q < 4; ++q) inside = inside && f[q] >= lo[q] && f[q] <= hi[q];
-    float v = inside ? mlp_row(sp, f, nullptr, nullptr) : 0.f;
+    float v = inside ? mlp_row(sp, f) : 0.f;
     s[r] = fminf(3.f, fmaxf(-3.f, v));
   }
 }
 
 static size_t grad_smem() {
-  return (size_t)(kMlpParams + 3 + 4 * GR * MH + GR * 4 + GR) * sizeof(float);
+  return (size_t)(GLOADS + MH * MH + 2 * MH * GP + GR * 4 + 4 * GR + GR) * sizeof(float);
 }
 
 void mlp_factors(System& s, const int* idx, int k, const double* theta, const double* rn,
@@ -382,8 +513,9 @@ pwh_status pwh_mlp_loss_grad(pwh_system* sys, const float* params, const float* 
     });
     PWH_CUDA(cudaMemsetAsync(grad_out, 0, kMlpParams * sizeof(float), s.stream));
     PWH_CUDA(cudaMemsetAsync(loss_out, 0, sizeof(float), s.stream));
-    const int blocks = (int)((rows + GR - 1) / GR);
-    k_mlp_grad<<<blocks, GR, grad_smem(), s.stream>>>(params, feats, y, w, rows, (float)(1.0 / wsum),
+    // persistent: two blocks per SM
+    const int blocks = (int)std::min<int64_t>(2 * 152, (rows + GR - 1) / GR);
+    k_mlp_grad<<<blocks, GT, grad_smem(), s.stream>>>(params, feats, y, w, rows, (float)(1.0 / wsum),
                                                       grad_out, loss_out);
     PWH_LAUNCH_CHECK();
   });
