@@ -284,8 +284,8 @@ static void cgemm_impl(System& s, bool conjA, int M, int N, int K, cx<TS> alpha,
   }
 }
 
-// FP64 products of at least kOzMinFlops go to the tensor cores as sliced
-// integer products (oz_gemm).
+// FP64 products of at least kOzMinFlops go to the tensor cores as integer
+// products by residues (oz_gemm).
 
 // The sliced tensor-core paths launch one block row per column of A (A^H B)
 // and of B along grid y, and K / 64 blocks along grid y of the A B slicing:

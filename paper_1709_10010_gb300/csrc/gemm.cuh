@@ -26,15 +26,16 @@ void cgemm_f32_simt(System& s, bool conjA, int M, int N, int K, double2 alpha, c
                     int64_t lda, const double2* B, int64_t ldb, double2 beta, double2* C,
                     int64_t ldc, cudaStream_t st);
 
-// Grow the sliced-product workspace for op(A) B of these sizes now (so that
+// Grow the residue workspace for op(A) B of these sizes now (so that
 // later products of at most this size allocate nothing).
 void oz_reserve(System& s, bool conjA, int M, int N, int K);
 // Products of at least this many flops (8 M N K) take oz_gemm in cgemm<double>.
 constexpr double kOzMinFlops = 2e8;
 
-// FP64-equivalent complex GEMM on the BF16 tensor cores (gemm_tc.cu): same
-// contract as cgemm<double>, results within FP64-level rounding (integer
-// slices of the operands, exact partial sums).
+// FP64-equivalent complex GEMM on the BF16 tensor cores (gemm_mod.cu): same
+// contract as cgemm<double>, results within FP64-level rounding (62-bit
+// integers, exact products by residues); a row of op(A) or column of B with an
+// infinity or NaN gives NaN.
 void oz_gemm(System& s, bool conjA, int M, int N, int K, double2 alpha, const double2* A,
              int64_t lda, const double2* B, int64_t ldb, double2 beta, double2* C, int64_t ldc,
              cudaStream_t st, const double* rowscale = nullptr);

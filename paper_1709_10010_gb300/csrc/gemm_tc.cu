@@ -28,25 +28,21 @@
 // timeout the kernel records PWH_ERR_TIMEOUT in a device word, stops issuing,
 // waits (bounded) for the copies it started, frees its tensor memory and
 // returns.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-#include <cuda_bf16.h>
-
 #include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "tc_ptx.cuh"
 
 namespace pwh {
 
-constexpr int TC_BM = 128, TC_BN = 256, TC_BK = 64, TC_STAGES = 4;
+constexpr int TC_BM = 128, TC_BN = 256, TC_STAGES = 4;
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;            // 16 KB
 constexpr int TC_B_BYTES = TC_BN * TC_BK * 2;            // 32 KB
 constexpr int TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;  // 48 KB
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 constexpr int TC_TMEM_COLS = 256;
-constexpr unsigned long long TC_WAIT_NS = 1000000000ull;  // 1 s
 
 struct TcArgs {
   int M, N;          // output rows (A rows) and columns (B rows)
@@ -58,125 +54,20 @@ struct TcArgs {
   int64_t ldv;
   int nb;
   int* err;          // device error word
-  // sliced operands: product t multiplies A segment oz_a[t] by B segment
-  // oz_b[t]; oz = 1: blockIdx.z = (K chunk, product), each partial one product
-  // (FP64-equivalent GEMM); oz = 2 (FP32-equivalent GEMM): blockIdx.z < z_rest
-  // takes kb_per_split blocks of products 1.., the others kps0 blocks of
-  // product 0
+  // sliced operands (FP32-equivalent GEMM, oz = 2): product t multiplies A
+  // segment oz_a[t] by B segment oz_b[t]; grid slices z < z_rest take
+  // kb_per_split blocks of products 1.., the others kps0 blocks of product 0
   int oz;
-  unsigned char oz_a[64], oz_b[64];
+  unsigned char oz_a[8], oz_b[8];
   int z_rest, kps0;
 };
 
-__device__ __forceinline__ uint32_t su32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(su32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait; also gives up early once *abort is raised by another role.
-__device__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  if (mbar_try(bar, parity)) return true;
-  const uint64_t t0 = gtimer();
-  while (true) {
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try(bar, parity)) return true;
-    if (abort && *abort) return false;
-    if (gtimer() - t0 > TC_WAIT_NS) return false;
-  }
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(su32(dst)),
-      "l"((uint64_t)map), "r"(x), "r"(y), "r"(su32(bar))
-      : "memory");
-}
-// Shared-memory matrix descriptor: K-major operand tile, rows of 128 bytes,
-// 128-byte swizzle, 8-row groups 1024 bytes apart (SBO), descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;                  // leading byte offset (unused here)
-  d |= (uint64_t)(1024 >> 4) << 32;        // stride byte offset
-  d |= (uint64_t)1 << 46;                  // version
-  d |= (uint64_t)2 << 61;                  // SWIZZLE_128B
-  return d;
-}
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          su32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// K blocks [kb0, kb_end) of grid slice z: sliced operands (oz = 1: z = chunk x
-// products + product; oz = 2: the long ranges of products 1.. first, then the
-// short ranges of product 0) or plain split-K ranges.
+// K blocks [kb0, kb_end) of grid slice z: sliced operands (oz = 2: the long
+// ranges of products 1.. first, then the short ranges of product 0) or plain
+// split-K ranges.
 __device__ __forceinline__ void tc_krange(const TcArgs& args, int z, int& kb0, int& kb_end) {
   const int kb_total = args.terms * args.kb_seg;
-  if (args.oz == 1) {
-    kb0 = (z % args.terms) * args.kb_seg + (z / args.terms) * args.kb_per_split;
-    kb_end = min(kb_total, kb0 + args.kb_per_split);
-  } else if (args.oz == 2 && z < args.z_rest) {
+  if (args.oz == 2 && z < args.z_rest) {
     kb0 = args.kb_seg + z * args.kb_per_split;
     kb_end = min(kb_total, kb0 + args.kb_per_split);
   } else if (args.oz == 2) {
@@ -505,43 +396,6 @@ __global__ void k_d_to_f32(const double2* __restrict__ src, int64_t n, float2* _
     dst[t] = make_float2((float)src[t].x, (float)src[t].y);
 }
 
-// ---------------------------------------------------------------- host -----
-static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static std::once_flag once;
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  std::call_once(once, [] {
-    cudaDriverEntryPointQueryResult q;
-    void* p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-  });
-  if (!fn) throw Error{PWH_ERR_CUDA, "cuTensorMapEncodeTiled unavailable"};
-  return fn;
-}
-
-// 2D BF16 K-major tensor map: rows x cols (cols contiguous, pitch in elements),
-// box 64 x box_rows, 128-byte swizzle, zero fill out of bounds.
-static CUtensorMap make_map(const void* base, int64_t rows, int64_t cols, int64_t pitch,
-                            int box_rows) {
-  CUtensorMap m;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)(pitch * 2)};
-  cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  if (((uintptr_t)base & 15) || ((pitch * 2) & 15))
-    throw Error{PWH_ERR_ARG, "tensor map base or pitch not 16-byte aligned"};
-  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims,
-                           strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) throw Error{PWH_ERR_CUDA, "cuTensorMapEncodeTiled failed"};
-  return m;
-}
-
-static int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
-
 // Operand geometry for this system (K segments padded to whole 64-wide blocks).
 struct TcGeom {
   int64_t seg1, pitch1;  // becp: K = npw
@@ -671,547 +525,6 @@ void nonlocal_mixed(System& s, int nb, const double2* psi, int64_t ldp, float2* 
   launch_tc(s, 1, ma2, mb2, a2, gm2, gn2, 1, st);
 }
 
-
-// ------------------------------------ FP64-equivalent complex GEMM (slices) ----
-// C = alpha op(A) B + beta C for FP64 (complex128) operands on the BF16 tensor
-// cores, accurate to about FP64 rounding: the error-free splitting of Ozaki et
-// al. (products of integer slices summed exactly).  Each real row r of an
-// operand (after the complex interleaving of the projector GEMM above) gets
-// the exponent e_r with max|x_r| < 2^e_r and is written as
-//     x = 2^e_r sum_{s < OZ_S} a_s 2^(-6 - 7 s),   a_s integers, |a_s| <= 64,
-// which BF16 holds exactly (balanced base-128 digits of the row-scaled value
-// as an integer).  A product a_s b_t is at most 2^12 and a sum of 4096 of
-// them at most 2^24, so every FP32 partial of a 4096-wide K chunk is an exact
-// integer (base-128 digits take one slice more than base-256 ones, 36 pairs
-// instead of 28, and write a third of the partials).  The partials of the
-// pairs with s + t <= OZ_G are summed in int64 by weight 2^(-7(s+t)) and
-// scaled once in FP64.  Dropped terms and slice truncation are below 2^-52 of
-// max|a| max|b| per elementary product.
-constexpr int OZ_S = 8;
-constexpr int OZ_G = OZ_S - 1;
-constexpr int OZ_PAIRS = (OZ_S * (OZ_S + 1)) / 2;  // pairs with s + t <= OZ_G
-constexpr int OZ_CHUNK_KB = 64;                    // 64-wide K blocks per exact partial
-static_assert(OZ_PAIRS <= 64, "pair table");
-__constant__ unsigned char c_oz_g[64];            // s + t of pair p
-
-// Slicing works on the IEEE bit patterns with integer arithmetic only (the
-// FP64 pipe of this GPU would make it the slowest step).  |x| as an unsigned
-// integer orders like |x|, so row maxima are integer maxima of these keys.
-__device__ __forceinline__ unsigned long long oz_key(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-}
-// exponent e with |x| < 2^e for the largest key of a row (0 for a zero row)
-__device__ __forceinline__ int oz_exp_of_key(unsigned long long k) {
-  if (k == 0) return 0;
-  const int eb = (int)(k >> 52);
-  return eb ? eb - 1022 : -1021;  // frexp exponent; subnormals lie below 2^-1022
-}
-// The OZ_S balanced base-128 digits of X = round(x 2^(55 - e)), |X| < 2^55:
-// x = 2^e sum_s a_s 2^(-6 - 7 s) up to 2^(e - 56), |a_s| <= 64, as BF16.
-__device__ __forceinline__ void oz_split(double x, int e, __nv_bfloat16* a) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int eb = (int)((bits >> 52) & 0x7ff);
-  const unsigned long long m = (bits & 0xfffffffffffffull) | (eb ? (1ull << 52) : 0ull);
-  const int sh = (eb ? eb : 1) - 1075 + 55 - e;  // X = m 2^sh
-  long long X;
-  if (sh >= 0) X = (long long)(m << sh);
-  else if (sh > -64) X = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
-  else X = 0;
-  if (bits >> 63) X = -X;
-#pragma unroll
-  for (int s = OZ_S - 1; s > 0; --s) {
-    const int d = (int)((X + 64) & 127) - 64;
-    a[s] = __int2bfloat16_rn(d);
-    X = (X - d) >> 7;
-  }
-  a[0] = __int2bfloat16_rn((int)X);
-}
-
-// Exponents of the rows 2j (real parts) and 2j+1 (imaginary parts) of the
-// interleaved operand whose row pair j is column j of X (K x J, ld): one block
-// per column.
-__global__ void k_oz_colexp(const double2* __restrict__ X, int64_t ld, int K, int* __restrict__ ex) {
-  __shared__ unsigned long long red[2][32];
-  const int j = blockIdx.x;
-  unsigned long long mr = 0, mi = 0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double2 v = X[(size_t)j * ld + k];
-    mr = max(mr, oz_key(v.x));
-    mi = max(mi, oz_key(v.y));
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, o));
-    mi = max(mi, __shfl_xor_sync(0xffffffffu, mi, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = mr;
-    red[1][threadIdx.x >> 5] = mi;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      mr = max(mr, red[0][w]);
-      mi = max(mi, red[1][w]);
-    }
-    ex[2 * j] = oz_exp_of_key(mr);
-    ex[2 * j + 1] = oz_exp_of_key(mi);
-  }
-}
-// Slices of that operand: row 2j+c, segment s holds a_s of (Re, Im) X[k][j]
-// at column s seg + k (zero for K <= k < seg).
-__global__ void k_oz_slice_cols(const double2* __restrict__ X, int64_t ld, int K, int seg,
-                                const int* __restrict__ ex, __nv_bfloat16* __restrict__ out,
-                                int64_t pitch) {
-  const int j = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= seg) return;
-  const double2 v = k < K ? X[(size_t)j * ld + k] : make_double2(0.0, 0.0);
-  __nv_bfloat16 ar[OZ_S], ai[OZ_S];
-  oz_split(v.x, ex[2 * j], ar);
-  oz_split(v.y, ex[2 * j + 1], ai);
-  __nv_bfloat16* r0 = out + (size_t)(2 * j) * pitch + k;
-  __nv_bfloat16* r1 = r0 + pitch;
-#pragma unroll
-  for (int s = 0; s < OZ_S; ++s) {
-    r0[(size_t)s * seg] = ar[s];
-    r1[(size_t)s * seg] = ai[s];
-  }
-}
-
-// Exponent of row m of the operand A2[m][2k+c] = (Re, Im) A[m][k] (A: M x K,
-// column-major, ld): one thread per row.
-__global__ void k_oz_rowexp(const double2* __restrict__ A, int64_t ld, int M, int K,
-                            int* __restrict__ ex) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M) return;
-  unsigned long long mx = 0;
-  for (int k = 0; k < K; ++k) {
-    const double2 v = A[(size_t)k * ld + m];
-    mx = max(mx, max(oz_key(v.x), oz_key(v.y)));
-  }
-  ex[m] = oz_exp_of_key(mx);
-}
-// Slices of A2: row m, segment s, column 2k+c (zero for 2K <= 2k+c < seg);
-// 32 x 32 tiles transposed through shared memory.
-__global__ void k_oz_slice_rows(const double2* __restrict__ A, int64_t ld, int M, int K, int seg,
-                                const int* __restrict__ ex, __nv_bfloat16* __restrict__ out,
-                                int64_t pitch) {
-  __shared__ double2 tile[32][33];
-  const int m0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
-  for (int t = threadIdx.x; t < 1024; t += blockDim.x) {
-    const int mm = t & 31, kk = t >> 5;
-    const int m = m0 + mm, k = k0 + kk;
-    tile[kk][mm] = (m < M && k < K) ? A[(size_t)k * ld + m] : make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < 1024; t += blockDim.x) {
-    const int kk = t & 31, mm = t >> 5;
-    const int m = m0 + mm, k = k0 + kk;
-    if (m >= M || 2 * k >= seg) continue;
-    const double2 v = tile[kk][mm];
-    const int e = ex[m];
-    __nv_bfloat16 ar[OZ_S], ai[OZ_S];
-    oz_split(v.x, e, ar);
-    oz_split(v.y, e, ai);
-    __nv_bfloat16* r = out + (size_t)m * pitch + 2 * k;
-#pragma unroll
-    for (int s = 0; s < OZ_S; ++s) {
-      __nv_bfloat162 p;
-      p.x = ar[s];
-      p.y = ai[s];
-      *(__nv_bfloat162*)(r + (size_t)s * seg) = p;
-    }
-  }
-}
-
-// B operand of the non-conjugated product: rows 2n, 2n+1 of
-//     B2[2n][2k] = Re, B2[2n][2k+1] = -Im, B2[2n+1][2k] = Im, B2[2n+1][2k+1] = Re
-// of B[k][n] (B: K x N, column-major, ld), both rows with the exponent of
-// max(|Re|, |Im|) over column n: one block per column.
-__global__ void k_oz_colexp_b2(const double2* __restrict__ B, int64_t ld, int K,
-                               int* __restrict__ ex) {
-  __shared__ unsigned long long red[32];
-  const int n = blockIdx.x;
-  unsigned long long mx = 0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double2 v = B[(size_t)n * ld + k];
-    mx = max(mx, max(oz_key(v.x), oz_key(v.y)));
-  }
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, red[w]);
-    ex[2 * n] = ex[2 * n + 1] = oz_exp_of_key(mx);
-  }
-}
-__global__ void k_oz_slice_b2(const double2* __restrict__ B, int64_t ld, int K, int seg,
-                              const int* __restrict__ ex, __nv_bfloat16* __restrict__ out,
-                              int64_t pitch) {
-  const int n = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (2 * k >= seg) return;
-  const double2 v = k < K ? B[(size_t)n * ld + k] : make_double2(0.0, 0.0);
-  const int e = ex[2 * n];
-  __nv_bfloat16 ar[OZ_S], ai[OZ_S];
-  oz_split(v.x, e, ar);
-  oz_split(v.y, e, ai);
-  __nv_bfloat16* r0 = out + (size_t)(2 * n) * pitch + 2 * k;
-  __nv_bfloat16* r1 = r0 + pitch;
-#pragma unroll
-  for (int s = 0; s < OZ_S; ++s) {
-    __nv_bfloat162 p0, p1;
-    p0.x = ar[s];
-    p0.y = __hneg(ai[s]);
-    p1.x = ai[s];
-    p1.y = ar[s];
-    *(__nv_bfloat162*)(r0 + (size_t)s * seg) = p0;
-    *(__nv_bfloat162*)(r1 + (size_t)s * seg) = p1;
-  }
-}
-
-// Exact accumulation of the integer partials of one real output: weights
-// 2^(-7g) folded into hi (g <= 3) and lo (g >= 4); value
-// 2^(e - 12) (hi 2^-21 + lo 2^-(7 OZ_G)).  At 161,235-wide K (40 chunks) both
-// stay below 2^53.
-struct OzAcc {
-  long long hi = 0, lo = 0;
-  // i: a sum of exact integer partials (each |v| <= 2^24) of weight 2^(-7g)
-  __device__ __forceinline__ void add_int(long long i, int g) {
-    if (g <= 3) hi += i * (1ll << (7 * (3 - g)));
-    else lo += i * (1ll << (7 * (OZ_G - g)));
-  }
-  __device__ __forceinline__ double value(int e) const {
-    return ldexp((double)hi, e - 12 - 21) + ldexp((double)lo, e - 12 - 7 * OZ_G);
-  }
-};
-
-// op(A) = A^H: complex (m, n) from the four real products of rows 2m, 2m+1 and
-// columns 2n, 2n+1 (Re = C[2m][2n] + C[2m+1][2n+1], Im = C[2m][2n+1] -
-// C[2m+1][2n]); part[z][n'][m'] with M' = 2M, N' = 2N, z = chunk * pairs + pair.
-__global__ void k_oz_reduce_cj(const float* __restrict__ part, int nz, int nchunk, int M, int N,
-                               const int* __restrict__ exa, const int* __restrict__ exb,
-                               const double* __restrict__ rowscale, double2 alpha, double2 beta,
-                               double2* __restrict__ C, int64_t ldc) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)M * N) return;
-  const int m = (int)(t % M), n = (int)(t / M);
-  const int64_t Mr = 2 * (int64_t)M, plane = Mr * 2 * (int64_t)N;
-  OzAcc q00, q10, q01, q11;
-  const float* p0 = part + (size_t)(2 * n) * Mr + 2 * m;      // (2m,2n), (2m+1,2n)
-  const float* p1 = part + (size_t)(2 * n + 1) * Mr + 2 * m;  // (2m,2n+1), (2m+1,2n+1)
-  const int npair = nz / nchunk;
-  for (int pr = 0; pr < npair; ++pr) {
-    const int g = c_oz_g[pr];
-    // the chunks of one pair share the weight: integer sums first, four
-    // partials in flight
-    long long s00 = 0, s10 = 0, s01 = 0, s11 = 0;
-    int c = 0;
-    for (; c + 3 < nchunk; c += 4) {
-      float2 a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const size_t z = (size_t)(c + u) * npair + pr;
-        a[u] = *(const float2*)(p0 + z * plane);
-        b[u] = *(const float2*)(p1 + z * plane);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        s00 += __float2int_rn(a[u].x);
-        s10 += __float2int_rn(a[u].y);
-        s01 += __float2int_rn(b[u].x);
-        s11 += __float2int_rn(b[u].y);
-      }
-    }
-    for (; c < nchunk; ++c) {
-      const size_t z = (size_t)c * npair + pr;
-      const float2 a = *(const float2*)(p0 + z * plane), b = *(const float2*)(p1 + z * plane);
-      s00 += __float2int_rn(a.x);
-      s10 += __float2int_rn(a.y);
-      s01 += __float2int_rn(b.x);
-      s11 += __float2int_rn(b.y);
-    }
-    q00.add_int(s00, g);
-    q10.add_int(s10, g);
-    q01.add_int(s01, g);
-    q11.add_int(s11, g);
-  }
-  const int ea0 = exa[2 * m], ea1 = exa[2 * m + 1], eb0 = exb[2 * n], eb1 = exb[2 * n + 1];
-  double re = q00.value(ea0 + eb0) + q11.value(ea1 + eb1);
-  double im = q01.value(ea0 + eb1) - q10.value(ea1 + eb0);
-  if (rowscale) {
-    re *= rowscale[m];
-    im *= rowscale[m];
-  }
-  double2 r = make_double2(alpha.x * re - alpha.y * im, alpha.x * im + alpha.y * re);
-  if (beta.x != 0.0 || beta.y != 0.0) {
-    const double2 c = C[(size_t)n * ldc + m];
-    r.x += beta.x * c.x - beta.y * c.y;
-    r.y += beta.x * c.y + beta.y * c.x;
-  }
-  C[(size_t)n * ldc + m] = r;
-}
-
-// op(A) = A: complex (m, n) = (C2[m][2n], C2[m][2n+1]); part[z][n'][m'] with
-// M' = M, N' = 2N.
-__global__ void k_oz_reduce_nn(const float* __restrict__ part, int nz, int nchunk, int M, int N,
-                               const int* __restrict__ exa, const int* __restrict__ exb,
-                               const double* __restrict__ rowscale, double2 alpha, double2 beta,
-                               double2* __restrict__ C, int64_t ldc) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)M * N) return;
-  const int m = (int)(t % M), n = (int)(t / M);
-  const int64_t plane = (int64_t)M * 2 * N;
-  OzAcc qr, qi;
-  const float* p0 = part + (size_t)(2 * n) * M + m;
-  const float* p1 = p0 + M;
-  const int npair = nz / nchunk;
-  if (nchunk == 1) {
-    // one chunk: every pair's partial in flight together
-#pragma unroll 9
-    for (int pr = 0; pr < OZ_PAIRS; ++pr) {
-      qr.add_int(__float2int_rn(p0[(size_t)pr * plane]), c_oz_g[pr]);
-      qi.add_int(__float2int_rn(p1[(size_t)pr * plane]), c_oz_g[pr]);
-    }
-  } else {
-    for (int pr = 0; pr < npair; ++pr) {
-      long long sr = 0, si = 0;
-      for (int c = 0; c < nchunk; ++c) {
-        const size_t z = (size_t)c * npair + pr;
-        sr += __float2int_rn(p0[z * plane]);
-        si += __float2int_rn(p1[z * plane]);
-      }
-      qr.add_int(sr, c_oz_g[pr]);
-      qi.add_int(si, c_oz_g[pr]);
-    }
-  }
-  const int e = exa[m] + exb[2 * n];
-  double re = qr.value(e), im = qi.value(e);
-  if (rowscale) {
-    re *= rowscale[m];
-    im *= rowscale[m];
-  }
-  double2 r = make_double2(alpha.x * re - alpha.y * im, alpha.x * im + alpha.y * re);
-  if (beta.x != 0.0 || beta.y != 0.0) {
-    const double2 c = C[(size_t)n * ldc + m];
-    r.x += beta.x * c.x - beta.y * c.y;
-    r.y += beta.x * c.y + beta.y * c.x;
-  }
-  C[(size_t)n * ldc + m] = r;
-}
-
-static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// Geometry and workspace of one sliced product.
-struct OzGeom {
-  int64_t Mr, Nr, seg, pitch;
-  int kb_seg, kbps, nchunk, nz;
-  size_t bytes_a, bytes_b, bytes_e, bytes_p;
-  size_t total() const { return bytes_a + bytes_b + bytes_e + bytes_p; }
-};
-static OzGeom oz_geom(bool conjA, int M, int N, int K) {
-  OzGeom g;
-  // real GEMM geometry: C' (Mr x Nr) = A' (Mr x Kr) B'^T, both K-major
-  g.Mr = conjA ? 2 * (int64_t)M : M;
-  g.Nr = 2 * (int64_t)N;
-  const int64_t Kr = conjA ? K : 2 * (int64_t)K;
-  g.seg = round_up(std::max<int64_t>(Kr, 1), TC_BK);
-  g.kb_seg = (int)(g.seg / TC_BK);
-  // K blocks per exact partial: at most OZ_CHUNK_KB (4096 wide) and dividing
-  // kb_seg; pad the segment to whole chunks when that costs little, else take
-  // a divisor of at least half a chunk
-  g.kbps = g.kb_seg;
-  if (g.kb_seg > OZ_CHUNK_KB) {
-    const int padc = (g.kb_seg + OZ_CHUNK_KB - 1) / OZ_CHUNK_KB * OZ_CHUNK_KB;
-    g.kbps = 0;
-    if ((padc - g.kb_seg) * 16 > g.kb_seg)
-      for (int d = OZ_CHUNK_KB; d >= OZ_CHUNK_KB / 2 && !g.kbps; --d)
-        if (g.kb_seg % d == 0) g.kbps = d;
-    if (!g.kbps) {
-      g.kb_seg = padc;
-      g.seg = (int64_t)g.kb_seg * TC_BK;
-      g.kbps = OZ_CHUNK_KB;
-    }
-  }
-  g.nchunk = g.kb_seg / g.kbps;
-  g.nz = OZ_PAIRS * g.nchunk;
-  g.pitch = OZ_S * g.seg;
-  g.bytes_a = align256((size_t)g.Mr * g.pitch * 2);
-  g.bytes_b = align256((size_t)g.Nr * g.pitch * 2);
-  g.bytes_e = align256((size_t)(g.Mr + g.Nr) * sizeof(int));
-  g.bytes_p = (size_t)g.nz * g.Mr * g.Nr * sizeof(float);
-  return g;
-}
-
-// The exact partials (OZ_PAIRS per K chunk, FP32, of the whole real output) are
-// bounded.  A product over many chunks first runs as K segments of whole
-// chunks, each added into C in FP64 (one more rounding per segment, no
-// operand sliced twice); a segment that still does not fit runs as pieces of
-// its larger output dimension, which give the same bits as the whole segment
-// (the exponents belong to single rows of op(A) and single columns of B).
-constexpr size_t kOzPartCap = (size_t)4 << 30;
-constexpr int kOzSegChunks = 8;
-
-struct OzSplit {
-  int kseg;      // complex K per segment
-  bool split_m;  // pieces of M (else of N)
-  int piece;     // rows or columns per piece
-};
-static OzSplit oz_split_of(bool conjA, int M, int N, int K) {
-  OzSplit sp{K, M >= N, M >= N ? M : N};
-  // at most kOzSegChunks 4096-wide real chunks a segment: the slices are
-  // stored [row][slice * seg + k], so the row pitch grows with the segment
-  // and one chunk's tiles spread over as many memory pages as there are rows
-  // (a 544 x 544 x 161,235 A^H B product ran its 25-chunk first segment at
-  // 0.57 ms a chunk and its 15-chunk second one at 0.36 ms)
-  const int kmax = (conjA ? 64 : 32) * OZ_CHUNK_KB * kOzSegChunks;
-  if (K > kmax) sp.kseg = kmax;
-  const OzGeom g = oz_geom(conjA, M, N, sp.kseg);
-  if (g.bytes_p <= kOzPartCap) return sp;
-  const size_t per_chunk = g.bytes_p / (size_t)g.nchunk;
-  if (g.nchunk > 1) {
-    // whole 4096-wide real chunks per segment (4096 complex K for A^H B,
-    // 2048 for A B, whose real K is 2K)
-    const int64_t c = std::max<int64_t>(1, (int64_t)(kOzPartCap / per_chunk));
-    const int64_t kc = conjA ? 64 * OZ_CHUNK_KB : 32 * OZ_CHUNK_KB;
-    if (c < g.nchunk) sp.kseg = (int)std::min<int64_t>(sp.kseg, c * kc);
-  }
-  const OzGeom gs = oz_geom(conjA, M, N, sp.kseg);
-  if (gs.bytes_p <= kOzPartCap) return sp;
-  const size_t per = gs.bytes_p / (size_t)sp.piece;  // partial bytes per row or column
-  const int64_t fit = (int64_t)(kOzPartCap / per) / 64 * 64;
-  sp.piece = (int)std::max<int64_t>(64, std::min<int64_t>(fit, sp.piece));
-  return sp;
-}
-
-void oz_reserve(System& s, bool conjA, int M, int N, int K) {
-  if (M <= 0 || N <= 0 || K <= 0) return;
-  const OzSplit sp = oz_split_of(conjA, M, N, K);
-  ensure(s.ws_oz, oz_geom(conjA, sp.split_m ? std::min(sp.piece, M) : M,
-                          sp.split_m ? N : std::min(sp.piece, N), sp.kseg)
-                      .total());
-}
-
-static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 alpha,
-                          const double2* A, int64_t lda, const double2* B, int64_t ldb,
-                          double2 beta, double2* C, int64_t ldc, cudaStream_t st,
-                          const double* rowscale);
-
-void oz_gemm(System& s, bool conjA, int M, int N, int K, double2 alpha, const double2* A,
-             int64_t lda, const double2* B, int64_t ldb, double2 beta, double2* C, int64_t ldc,
-             cudaStream_t st, const double* rowscale) {
-  if (M <= 0 || N <= 0) return;
-  const OzSplit sp = oz_split_of(conjA, M, N, K);
-  for (int k0 = 0; k0 == 0 || k0 < K; k0 += sp.kseg) {
-    const int kk = std::min(sp.kseg, K - k0);
-    // K rows k0.. of B and of A (A^H), or K columns k0.. of A
-    const double2* Ak = A + (conjA ? (int64_t)k0 : (int64_t)k0 * lda);
-    const double2* Bk = B + k0;
-    const double2 bk = k0 == 0 ? beta : make_double2(1, 0);
-    if (sp.split_m) {
-      // rows m0.. of C: columns m0.. of A (A^H) or rows m0.. of A
-      for (int m0 = 0; m0 < M; m0 += sp.piece)
-        oz_gemm_piece(s, conjA, std::min(sp.piece, M - m0), N, kk, alpha,
-                      Ak + (conjA ? (int64_t)m0 * lda : (int64_t)m0), lda, Bk, ldb, bk, C + m0,
-                      ldc, st, rowscale ? rowscale + m0 : nullptr);
-    } else {
-      for (int n0 = 0; n0 < N; n0 += sp.piece)
-        oz_gemm_piece(s, conjA, M, std::min(sp.piece, N - n0), kk, alpha, Ak, lda,
-                      Bk + (int64_t)n0 * ldb, ldb, bk, C + (int64_t)n0 * ldc, ldc, st, rowscale);
-    }
-  }
-}
-
-static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 alpha,
-                          const double2* A, int64_t lda, const double2* B, int64_t ldb,
-                          double2 beta, double2* C, int64_t ldc, cudaStream_t st,
-                          const double* rowscale) {
-  static std::once_flag once;
-  static unsigned char pa[64], pb[64];
-  std::call_once(once, [] {
-    unsigned char g[64] = {};
-    // pairs by A slice, then B slice: consecutive grid slices share an A
-    // slice, so one K chunk needs one A slice and its B slices in L2 at a time
-    int p = 0;
-    for (int sa = 0; sa <= OZ_G; ++sa)
-      for (int sb = 0; sa + sb <= OZ_G; ++sb) {
-        pa[p] = (unsigned char)sa;
-        pb[p] = (unsigned char)sb;
-        g[p] = (unsigned char)(sa + sb);
-        ++p;
-      }
-    cudaMemcpyToSymbol(c_oz_g, g, sizeof(g));
-    cudaFuncSetAttribute(k_tc_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-  });
-  const OzGeom gg = oz_geom(conjA, M, N, K);
-  const int64_t Mr = gg.Mr, Nr = gg.Nr, seg = gg.seg;
-  const int kb_seg = gg.kb_seg, kbps = gg.kbps, nchunk = gg.nchunk, nz = gg.nz;
-  const int64_t pitch = gg.pitch;
-  const size_t bytes_a = gg.bytes_a, bytes_b = gg.bytes_b, bytes_e = gg.bytes_e;
-  ensure(s.ws_oz, gg.total());
-  char* base = s.ws_oz.p;
-  __nv_bfloat16* pA = (__nv_bfloat16*)base;
-  __nv_bfloat16* pB = (__nv_bfloat16*)(base + bytes_a);
-  int* exa = (int*)(base + bytes_a + bytes_b);
-  int* exb = exa + Mr;
-  float* part = (float*)(base + bytes_a + bytes_b + bytes_e);
-
-  // timed as its own family: the work is the real BF16 tensor-core GEMM of
-  // all slice pairs (2 Mr Nr Kr per pair)
-  TimedScope ts(s, KF_GEMM_OZ, st, 2.0 * OZ_PAIRS * (double)Mr * Nr * (double)seg,
-                2.0 * OZ_PAIRS * ((double)Mr + Nr) * seg + 8.0 * nz * (double)Mr * Nr);
-  // slices of op(A) and B
-  if (conjA) {
-    k_oz_colexp<<<M, 256, 0, st>>>(A, lda, K, exa);
-    PWH_LAUNCH_CHECK();
-    k_oz_slice_cols<<<dim3((unsigned)((seg + 255) / 256), M), 256, 0, st>>>(A, lda, K, (int)seg, exa,
-                                                                            pA, pitch);
-    PWH_LAUNCH_CHECK();
-    k_oz_colexp<<<N, 256, 0, st>>>(B, ldb, K, exb);
-    PWH_LAUNCH_CHECK();
-    k_oz_slice_cols<<<dim3((unsigned)((seg + 255) / 256), N), 256, 0, st>>>(B, ldb, K, (int)seg, exb,
-                                                                            pB, pitch);
-    PWH_LAUNCH_CHECK();
-  } else {
-    k_oz_rowexp<<<(M + 255) / 256, 256, 0, st>>>(A, lda, M, K, exa);
-    PWH_LAUNCH_CHECK();
-    k_oz_slice_rows<<<dim3((M + 31) / 32, (unsigned)((seg / 2 + 31) / 32)), 256, 0, st>>>(
-        A, lda, M, K, (int)seg, exa, pA, pitch);
-    PWH_LAUNCH_CHECK();
-    k_oz_colexp_b2<<<N, 256, 0, st>>>(B, ldb, K, exb);
-    PWH_LAUNCH_CHECK();
-    k_oz_slice_b2<<<dim3((unsigned)((seg / 2 + 255) / 256), N), 256, 0, st>>>(B, ldb, K, (int)seg,
-                                                                              exb, pB, pitch);
-    PWH_LAUNCH_CHECK();
-  }
-  // every slice pair, every K chunk: exact FP32 partials on the tensor cores
-  CUtensorMap ma = make_map(pA, Mr, pitch, pitch, TC_BM);
-  CUtensorMap mb = make_map(pB, Nr, pitch, pitch, TC_BN);
-  TcArgs a{};
-  a.M = (int)Mr;
-  a.N = (int)Nr;
-  a.kb_seg = kb_seg;
-  a.terms = OZ_PAIRS;
-  a.kb_per_split = kbps;
-  a.part = part;
-  a.err = device_error_word(s);
-  a.oz = 1;
-  for (int p = 0; p < OZ_PAIRS; ++p) {
-    a.oz_a[p] = pa[p];
-    a.oz_b[p] = pb[p];
-  }
-  dim3 grid((unsigned)((Mr + TC_BM - 1) / TC_BM), (unsigned)((Nr + TC_BN - 1) / TC_BN), nz);
-  tc_launch<0>(ma, mb, a, grid, st);
-  PWH_LAUNCH_CHECK();
-  const int64_t tot = (int64_t)M * N;
-  if (conjA)
-    k_oz_reduce_cj<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(part, nz, nchunk, M, N, exa, exb,
-                                                                  rowscale, alpha, beta, C, ldc);
-  else
-    k_oz_reduce_nn<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(part, nz, nchunk, M, N, exa, exb,
-                                                                  rowscale, alpha, beta, C, ldc);
-  PWH_LAUNCH_CHECK();
-}
 
 // ------------------------------------- FP32-equivalent GEMM (3 BF16 slices) --
 // Each real operand value, rounded to FP32, is the exact sum of three BF16
