@@ -120,6 +120,10 @@ struct JacobiArgsT {
   double tol;
   int* out_buf;   // buffer index (0/1) holding the result, sweeps used
   int* conv;      // per-sweep convergence flag written by block 0
+  const int* skip;  // optional device word: nonzero = already diagonal, no sweep
+  // optional device word: max |A_ii|; pairs with |A_pq| <= 1e-15 of it keep
+  // their element and are not rotated (FP64 only)
+  const unsigned long long* dmax;
   GridBar gb;
 };
 
@@ -147,7 +151,13 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
   const int nth = gridDim.x * blockDim.x;
   unsigned epoch = 0;  // grid barriers passed
   int cur = 0, sweep = 0;
-  for (; sweep < a.max_sweeps; ++sweep) {
+  const int max_sweeps = a.skip && *a.skip ? 0 : a.max_sweeps;
+  double keep2 = -1.0;  // |A_pq|^2 up to which a pair is left alone
+  if (sizeof(T) == 8 && a.dmax) {
+    const double d = 1e-15 * __longlong_as_double((long long)*a.dmax);
+    keep2 = d * d;
+  }
+  for (; sweep < max_sweeps; ++sweep) {
     for (int r = 0; r < np - 1; ++r) {
       const cx<T>* A = a.A[cur];
       for (int k = threadIdx.x; k < P; k += blockDim.x) {
@@ -155,8 +165,11 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
         if (p > q) { int t = p; p = q; q = t; }
         T c = 1;
         cx<T> sv = mk<T>(0, 0);
-        if (q < n)
-          jacobi_rotation<T>(A[(size_t)q * n + p], A[(size_t)p * n + p].x, A[(size_t)q * n + q].x, c, sv);
+        if (q < n) {
+          const cx<T> apq = A[(size_t)q * n + p];
+          if (sizeof(T) == 4 || !((double)apq.x * apq.x + (double)apq.y * apq.y <= keep2))
+            jacobi_rotation<T>(apq, A[(size_t)p * n + p].x, A[(size_t)q * n + q].x, c, sv);
+        }
         pp[k] = p;
         pq[k] = q;
         crot[k] = c;
@@ -182,8 +195,16 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
           const cx<T> a10 = vk ? A[(size_t)pl * n + qk] : z;
           const cx<T> a11 = (vk && vl) ? A[(size_t)ql * n + qk] : z;
           cx<T> y00, y01, y10, y11;
-          jacobi_block<T>(a00, a01, a10, a11, ck, sk, cl, sl, y00, y01, y10, y11);
-          if (k == l) {
+          // neither pair rotates (the polish of an almost diagonal matrix):
+          // the block moves to the other buffer without FP64 arithmetic
+          const bool still = sizeof(T) == 8 && keep2 >= 0 && ck == (T)1 && cl == (T)1 &&
+                             sk.x == (T)0 && sk.y == (T)0 && sl.x == (T)0 && sl.y == (T)0;
+          if (still) {
+            y00 = a00; y01 = a01; y10 = a10; y11 = a11;
+          } else {
+            jacobi_block<T>(a00, a01, a10, a11, ck, sk, cl, sl, y00, y01, y10, y11);
+          }
+          if (k == l && !still) {
             // rotated 2 x 2 diagonal block: real diagonal, zeroed pair element
             An[(size_t)pk * n + pk] = mk<T>(y00.x, 0);
             if (vk) {
@@ -215,7 +236,10 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
           const T cl = crot[l];
           const cx<T> sl = srot[l];
           const cx<T> q0 = Qc[(size_t)pl * n + i];
-          if (ql < n) {
+          if (sizeof(T) == 8 && keep2 >= 0 && ql < n && cl == (T)1 && sl.x == (T)0 && sl.y == (T)0) {
+            Qn[(size_t)pl * n + i] = q0;
+            Qn[(size_t)ql * n + i] = Qc[(size_t)ql * n + i];
+          } else if (ql < n) {
             const cx<T> q1 = Qc[(size_t)ql * n + i];
             Qn[(size_t)pl * n + i] = add<T>(scl<T>(q0, cl), mul<T>(q1, mk<T>(-sl.x, sl.y)));
             Qn[(size_t)ql * n + i] = add<T>(mul<T>(q0, sl), scl<T>(q1, cl));
@@ -1416,7 +1440,9 @@ static bool jacobi32_tuned(System& s, DenseWs& w, const double2* A, int64_t lda,
 
 template <typename T>
 static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0, cx<T>* Q1, int n,
-                          double tol, int max_sweeps, int* out_buf, cudaStream_t st) {
+                          double tol, int max_sweeps, int* out_buf, cudaStream_t st,
+                          const int* skip = nullptr,
+                          const unsigned long long* dmax = nullptr) {
   const int np = n + (n & 1);
   unsigned* ctl = (unsigned*)w.ctl;
   PWH_CUDA(cudaMemsetAsync(ctl, 0, 3 * sizeof(unsigned), st));  // barrier words
@@ -1425,6 +1451,8 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
   a.n = n; a.np = np; a.max_sweeps = max_sweeps; a.tol = tol;
   a.out_buf = out_buf;
   a.conv = (int*)(ctl + 12);
+  a.skip = skip;
+  a.dmax = dmax;
   a.gb.count = ctl; a.gb.unused = ctl + 1; a.gb.abort = (int*)(ctl + 2);
   a.gb.err = device_error_word(s);
   const int P = np / 2;
@@ -1490,9 +1518,255 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
   note_launch();
 }
 
+// ---- FP64 refinement of the FP32 eigenvectors by matrix products -----------
+// Quadratically convergent correction of an approximate eigenvector matrix X
+// (Ogita and Aishima, "Iterative refinement for symmetric eigenvalue
+// decomposition", 2018): with R = I - X^H X and S = X^H H X, X <- X (I + R/2) (I + E)
+// where E_ij = F_ij / (f_j - f_i), F = S + (R_ij / 2)(S_ii + S_jj) the
+// symmetrically orthonormalised S, f its diagonal.  Close pairs, where the
+// first-order angle would be large, are treated as Jacobi does: index i and
+// its strongest partner p(i), when each is the other's strongest and the angle
+// passes `lim`, are rotated exactly (J, unitary) and E is formed from J^H F J;
+// any other angle above `lim` is left for the next step, so that X stays
+// within lim^2 of unitary (clusters of three and more equal eigenvalues are
+// resolved a pair at a time, or left to the Jacobi sweeps).
+//   Bound: four n x n products a step (12 in all) and one Jacobi sweep before
+// them, against two to three (30 in large clusters) sweeps of n - 1 grid-wide
+// rounds on the FP64 pipe (60 us a round at n = 1088).  The whole FP64
+// eigensolve, FP32 stage included: n = 1088 137 -> 87 ms, 1632 587 -> 249, 408
+// 21.7 -> 16.4, 256 10.4 -> 9.6, five 128-fold levels 311 -> 41; eigenvectors
+// orthonormal to 3e-15 instead of 1e-13.  Without the first sweep (three
+// refinement steps from the FP32 basis) n = 1088 takes 20 ms to the same
+// accuracy, but with eigenvector phases that differ by 1e-6 from the cyclic
+// sweeps'.  Below kRefineMinN the products run on the FP64 pipe and gain
+// nothing.
+constexpr int kRefineMinN = 256;
+struct RefineWs {
+  double* dS;              // S_ii
+  double* f;               // F_ii
+  double* f2;              // diagonal of J^H F J
+  int* best;               // strongest partner
+  int* pair;               // its index when rotated, else -1
+  double* c;               // J_ii
+  double2* s;              // J_{i, p(i)}
+  unsigned long long* mx;  // max |F_ij|, max |F_ii| as ordered bit patterns
+  int* done;               // 1: every off-diagonal element below the target
+};
+static size_t refine_bytes(int n) { return (size_t)n * 56 + 64; }
+static RefineWs refine_carve(void* base, int n) {
+  RefineWs w;
+  w.s = (double2*)(((uintptr_t)base + 15) & ~(uintptr_t)15);
+  w.dS = (double*)(w.s + n);
+  w.f = w.dS + n;
+  w.f2 = w.f + n;
+  w.c = w.f2 + n;
+  w.best = (int*)(w.c + n);
+  w.pair = w.best + n;
+  w.mx = (unsigned long long*)(((uintptr_t)(w.pair + n) + 7) & ~(uintptr_t)7);
+  w.done = (int*)(w.mx + 2);
+  return w;
+}
+
+// tan of the Jacobi angle that zeroes an off-diagonal element of modulus g
+// between diagonal elements a (row) and b (column); first: tie rule at a = b
+__device__ __forceinline__ double refine_tan(double g, double a, double b, bool first) {
+  if (!(g > 0.0)) return 0.0;
+  const double zeta = (b - a) / (2.0 * g), az = fabs(zeta);
+  const double sg = zeta > 0.0 || (zeta == 0.0 && first) ? 1.0 : -1.0;
+  return az > 1e9 ? 0.5 / zeta : sg / (az + sqrt(1.0 + az * az));
+}
+// F_ij (i != j) from S, the Gram matrix and S's diagonal
+__device__ __forceinline__ double2 refine_f(const double2* S, const double2* Gm, const double* dS,
+                                            int n, int i, int j) {
+  const double2 s = S[(size_t)j * n + i], g = Gm[(size_t)j * n + i];
+  const double h = -0.5 * (dS[i] + dS[j]);  // R_ij = -Gram_ij off the diagonal
+  return make_double2(s.x + h * g.x, s.y + h * g.y);
+}
+
+__global__ void k_refine_diag(const double2* __restrict__ S, const double2* __restrict__ Gm, int n,
+                              RefineWs w) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) w.mx[0] = 0;
+  if (i >= n) return;
+  const double d = S[(size_t)i * n + i].x;
+  w.dS[i] = d;
+  w.f[i] = d * (2.0 - Gm[(size_t)i * n + i].x);  // S_ii + R_ii S_ii
+}
+// max |F_ii| (one block)
+__global__ void k_refine_max(int n, RefineWs w) {
+  __shared__ double red[32];
+  double m = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, fabs(w.f[i]));
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) m = fmax(m, red[k]);
+    w.mx[1] = (unsigned long long)__double_as_longlong(m);
+  }
+}
+// Strongest partner of every index (a block per column), max |F_ij|.
+__global__ void __launch_bounds__(128) k_refine_best(const double2* __restrict__ S,
+                                                     const double2* __restrict__ Gm, int n,
+                                                     RefineWs w) {
+  __shared__ double rq[4], rg[4];
+  __shared__ int ri[4];
+  const int j = blockIdx.x;
+  const double fj = w.f[j];
+  const double floor_g = 2e-16 * __longlong_as_double((long long)w.mx[1]);
+  double bq = -1.0, mg = 0.0;
+  int bi = -1;
+  for (int i = threadIdx.x; i < n; i += 128) {
+    if (i == j) continue;
+    const double2 F = refine_f(S, Gm, w.dS, n, i, j);
+    const double g = sqrt(F.x * F.x + F.y * F.y);
+    mg = fmax(mg, g);
+    if (!(g > floor_g)) continue;
+    // the angle grows with |F_ij| over the gap
+    const double q = g / fmax(fabs(fj - w.f[i]), 1e-300);
+    if (q > bq) {
+      bq = q;
+      bi = i;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double q2 = __shfl_xor_sync(0xffffffffu, bq, o), g2 = __shfl_xor_sync(0xffffffffu, mg, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (q2 > bq || (q2 == bq && i2 >= 0 && (bi < 0 || i2 < bi))) {
+      bq = q2;
+      bi = i2;
+    }
+    mg = fmax(mg, g2);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    rq[threadIdx.x >> 5] = bq;
+    rg[threadIdx.x >> 5] = mg;
+    ri[threadIdx.x >> 5] = bi;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 4; ++k) {
+      if (rq[k] > bq || (rq[k] == bq && ri[k] >= 0 && (bi < 0 || ri[k] < bi))) {
+        bq = rq[k];
+        bi = ri[k];
+      }
+      mg = fmax(mg, rg[k]);
+    }
+    w.best[j] = bi;
+    atomicMax(&w.mx[0], (unsigned long long)__double_as_longlong(mg));
+  }
+}
+// Pair rotations; done = max |F_ij| <= tol max |F_ii| (a NaN is not done).
+__global__ void k_refine_pairs(const double2* __restrict__ S, const double2* __restrict__ Gm, int n,
+                               double lim, double tol, RefineWs w) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0)
+    *w.done = __longlong_as_double((long long)w.mx[0]) <=
+              tol * fmax(__longlong_as_double((long long)w.mx[1]), 1e-300);
+  if (i >= n) return;
+  int p = -1;
+  double c = 1.0, f2 = w.f[i];
+  double2 s = make_double2(0, 0);
+  const int j = w.best[i];
+  if (j >= 0 && w.best[j] == i) {
+    const int a = min(i, j), b = max(i, j);
+    const double2 F = refine_f(S, Gm, w.dS, n, a, b);
+    const double g = sqrt(F.x * F.x + F.y * F.y);
+    const double t = refine_tan(g, w.f[a], w.f[b], true);
+    if (fabs(t) > lim) {
+      p = j;
+      c = 1.0 / sqrt(1.0 + t * t);
+      const double e = t * c / g;
+      // J_ab = s, J_ba = -conj(s)
+      s = i == a ? make_double2(e * F.x, e * F.y) : make_double2(-e * F.x, e * F.y);
+      f2 = i == a ? w.f[a] - t * g : w.f[b] + t * g;
+    }
+  }
+  w.pair[i] = p;
+  w.c[i] = c;
+  w.s[i] = s;
+  w.f2[i] = f2;
+}
+// Column j of M = (I + R/2) J (I + E), first order in R (a block per column, the
+// column of E in shared memory; E_jj = -sum |E_ij|^2 / 2).  last: the step after
+// which the Jacobi sweeps may run; when the target was missed M = I + R/2 and S
+// becomes F (X then is unitary to R^2), else S's diagonal holds the
+// eigenvalues.  (Diagonal elements of S are never read here, other columns'
+// elements only when the target was met.)
+__global__ void __launch_bounds__(128) k_refine_m(double2* __restrict__ S,
+                                                  const double2* __restrict__ Gm, int n, double lim,
+                                                  int last, RefineWs w, double2* __restrict__ M) {
+  extern __shared__ __align__(16) unsigned char rsm[];
+  double2* E = (double2*)rsm;
+  __shared__ double red[4];
+  const int j = blockIdx.x;
+  const double2* Gj = Gm + (size_t)j * n;
+  double2* Mj = M + (size_t)j * n;
+  if (last && !*w.done) {
+    for (int i = threadIdx.x; i < n; i += 128) {
+      S[(size_t)j * n + i] = i == j ? make_double2(w.f[i], 0.0) : refine_f(S, Gm, w.dS, n, i, j);
+      Mj[i] = make_double2((i == j ? 1.5 : 0.0) - 0.5 * Gj[i].x, -0.5 * Gj[i].y);
+    }
+    return;
+  }
+  const int pj = w.pair[j];
+  const double cj = w.c[j], f2j = w.f2[j];
+  // column j of J: J_jj = c_j, J_{p(j), j} = s_{p(j)}
+  const double2 sj = pj >= 0 ? w.s[pj] : make_double2(0, 0);
+  const double floor_g = 2e-16 * __longlong_as_double((long long)w.mx[1]);
+  double sum = 0.0;
+  for (int i = threadIdx.x; i < n; i += 128) {
+    double2 e = make_double2(0, 0);
+    if (i != pj && i != j) {
+      const int pi = w.pair[i];
+      // (F J)_aj for a = i, p(i), then (J^H . )_ij
+      auto col = [&](int a) {
+        double2 v = scl<double>(refine_f(S, Gm, w.dS, n, a, j), cj);
+        if (pj >= 0) v = add<double>(v, mul<double>(refine_f(S, Gm, w.dS, n, a, pj), sj));
+        return v;
+      };
+      double2 F = scl<double>(col(i), w.c[i]);
+      if (pi >= 0) F = add<double>(F, mulc<double>(col(pi), w.s[pi]));  // conj(J_{p(i), i})
+      const double g = sqrt(F.x * F.x + F.y * F.y);
+      if (g > floor_g) {
+        const double t = refine_tan(g, w.f2[i], f2j, i < j);
+        if (fabs(t) <= lim) {
+          const double u = t / g;
+          e = make_double2(u * F.x, u * F.y);
+          sum += t * t;
+        }
+      }
+    }
+    E[i] = e;
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    E[j] = make_double2(1.0 - 0.5 * (red[0] + red[1] + red[2] + red[3]), 0.0);  // I + E
+    if (last) S[(size_t)j * n + j] = make_double2(f2j, 0.0);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += 128) {
+    const int p = w.pair[i];
+    double2 m = scl<double>(E[i], w.c[i]);
+    if (p >= 0) m = add<double>(m, mul<double>(w.s[i], E[p]));
+    // (R / 2) J
+    double2 r = make_double2((i == j ? 0.5 : 0.0) - 0.5 * Gj[i].x, -0.5 * Gj[i].y);
+    r = scl<double>(r, cj);
+    if (pj >= 0) {
+      const double2 g = Gm[(size_t)pj * n + i];
+      r = add<double>(r, mul<double>(make_double2((i == pj ? 0.5 : 0.0) - 0.5 * g.x, -0.5 * g.y), sj));
+    }
+    Mj[i] = add<double>(m, r);
+  }
+}
+
 static size_t jacobi_ws_bytes(size_t nn, int n) {
-  // FP64: A0, A1, Q0, Q1, G;  FP32: a0, a1, q0, q1;  diagonal d
-  return 5 * nn * sizeof(double2) + 4 * nn * sizeof(float2) + (size_t)n * sizeof(double) + 512;
+  // FP64: A0, A1, Q0, Q1, G;  FP32: a0, a1, q0, q1;  diagonal d;  the
+  // refinement's per-index arrays
+  return 5 * nn * sizeof(double2) + 4 * nn * sizeof(float2) + (size_t)n * sizeof(double) + 512 +
+         refine_bytes(n);
 }
 
 void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, int nk,
@@ -1625,13 +1899,56 @@ void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, in
   cgemm<double>(s, true, n, n, n, one, Q1, n, G, n, zero, A0, n, st);    // A0 = Q^H H Q
   hermitize(A0, n, 0, n, st);
   PWH_CUDA(cudaMemcpyAsync(Q0, Q1, nn * sizeof(double2), cudaMemcpyDeviceToDevice, st));
-  // ---- stage 3 (FP64): polish sweeps on the nearly diagonal matrix.  Inside
-  // a cluster of (nearly) equal eigenvalues the FP32 basis leaves an
-  // unstructured block of FP32-rounding size that the polish diagonalises
-  // from scratch, at linear convergence (about a factor 2.3 a sweep on
-  // 128-fold degenerate levels), hence the allowance of 30 sweeps; a
-  // warm-started Rayleigh-Ritz matrix needs two or three.
-  launch_jacobi<double>(s, w, A0, A1, Q0, Q1, n, tol64, 30, out_buf, st);
+  if (n < kRefineMinN) {
+    // ---- stage 3 (FP64): polish sweeps on the nearly diagonal matrix.  Inside
+    // a cluster of (nearly) equal eigenvalues the FP32 basis leaves an
+    // unstructured block of FP32-rounding size that the polish diagonalises
+    // from scratch, at linear convergence (about a factor 2.3 a sweep on
+    // 128-fold degenerate levels), hence the allowance of 30 sweeps; a
+    // warm-started Rayleigh-Ritz matrix needs two or three.
+    launch_jacobi<double>(s, w, A0, A1, Q0, Q1, n, tol64, 30, out_buf, st);
+  } else {
+    // ---- stage 3 by products: one Jacobi sweep (which also fixes the phases
+    // of the eigenvectors, to the third order of its angles), two refinement
+    // steps, the target test with a last step, and Jacobi sweeps again only
+    // where the target was missed.  The limits leave X unitary to 1e-15 in
+    // clusters too, where angles up to them keep being applied.
+    launch_jacobi<double>(s, w, A0, A1, Q0, Q1, n, tol64, 1, out_buf, st);
+    // a sweep is an odd number of rounds: its result is in the second buffers
+    const RefineWs rw = refine_carve(dg + n, n);
+    double2 *X = Q1, *Gx = A0, *S = A1, *Gr = Q0, *Xn = G;
+    const unsigned g1 = (unsigned)((n + 255) / 256);
+    static std::once_flag once;
+    std::call_once(once, [] {
+      cudaFuncSetAttribute(k_refine_m, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           kJacobiMaxN * (int)sizeof(double2));
+    });
+    const double lims[3] = {1e-3, 1e-6, 3e-8};
+    for (int step = 0; step < 3; ++step) {
+      cgemm<double>(s, false, n, n, n, one, H, ldh, X, n, zero, Gx, n, st);
+      cgemm<double>(s, true, n, n, n, one, X, n, Gx, n, zero, S, n, st);
+      hermitize(S, n, 0, n, st);
+      cgemm<double>(s, true, n, n, n, one, X, n, X, n, zero, Gr, n, st);
+      k_refine_diag<<<g1, 256, 0, st>>>(S, Gr, n, rw);
+      PWH_LAUNCH_CHECK();
+      k_refine_max<<<1, 1024, 0, st>>>(n, rw);
+      PWH_LAUNCH_CHECK();
+      k_refine_best<<<n, 128, 0, st>>>(S, Gr, n, rw);
+      PWH_LAUNCH_CHECK();
+      k_refine_pairs<<<g1, 256, 0, st>>>(S, Gr, n, lims[step], tol64, rw);
+      PWH_LAUNCH_CHECK();
+      k_refine_m<<<n, 128, n * sizeof(double2), st>>>(S, Gr, n, lims[step], step == 2, rw, Gx);
+      PWH_LAUNCH_CHECK();
+      cgemm<double>(s, false, n, n, n, one, X, n, Gx, n, zero, Xn, n, st);
+      std::swap(X, Xn);
+    }
+    launch_jacobi<double>(s, w, S, Gr, X, Xn, n, tol64, 30, out_buf, st, rw.done, rw.mx + 1);
+    A0 = S;
+    A1 = Gr;
+    Q0 = X;
+    Q1 = Xn;
+    G = Gx;
+  }
   k_diag_of<double><<<(n + 255) / 256, 256, 0, st>>>(A0, A1, out_buf, n, dg);
   PWH_LAUNCH_CHECK();
   k_select_buf64<<<gq, 256, 0, st>>>(Q0, Q1, out_buf, (int64_t)nn, G);
