@@ -7,6 +7,7 @@
 #pragma once
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -99,6 +100,62 @@ constexpr int fft_factor(int n) {
   return best;
 }
 
+// Whether T is double-float: its arithmetic is the passes' limit, so it takes
+// the factorisation with the fewest products.  The other types keep theirs.
+struct df;
+template <typename T> constexpr bool is_df = std::is_same<T, df>::value;
+
+constexpr int gcd_of(int a, int b) { return b ? gcd_of(b, a % b) : a; }
+constexpr int inv_mod(int a, int m) {
+  for (int x = 0; x < m; ++x)
+    if (a * x % m == 1 % m) return x;
+  return 0;
+}
+// a factor N1 of N with N1 < N2 = N / N1 <= 16 coprime, as balanced as possible; 1
+// if there is none (50 and 96 of the compiled sizes)
+constexpr int coprime_factor(int n) {
+  int best = 1;
+  for (int d = 2; d <= 16; ++d)
+    if (n % d == 0 && n / d <= 16 && d < n / d && gcd_of(d, n / d) == 1) best = d;
+  return best;
+}
+// N = N1 N2 in two passes.  Four-step: element N2 n1 + n2 in, k1 + N1 k2 out,
+// twiddles w^(n2 k1) between.  Coprime factors in double-float (prime-factor
+// algorithm, Good 1958 and Thomas 1963): element (N2 n1 + N1 n2) mod N in,
+// (N2 t1 k1 + N1 t2 k2) mod N out with t1 = N2^-1 mod N1, t2 = N1^-1 mod N2, and no
+// twiddles.  idx_a(n1, n2) is the input element and the place of (k1 = n1, n2)
+// between the passes (the same set for fixed n2: pass 1 works in place);
+// idx_b(k1, k2) the output.  Forward transforms of the rows run with the two
+// maps exchanged.
+template <typename T, int N> struct Fac {
+  static constexpr bool pfa = is_df<T> && coprime_factor(N) > 1;
+  static constexpr int N1 = pfa ? coprime_factor(N) : fft_factor(N), N2 = N / N1;
+  static_assert(N1 > 1 && N1 <= 16 && N2 <= 16, "factor");
+  static constexpr int A = pfa ? N2 * inv_mod(N2, N1) % N : 1;
+  static constexpr int B = pfa ? N1 * inv_mod(N1, N2) % N : N1;
+  __device__ static __forceinline__ int wrap(int i) { return i >= N ? i - N : i; }
+  __device__ static __forceinline__ int idx_a(int n1, int n2) {
+    if constexpr (pfa) return wrap(N1 * n2 + N2 * n1);
+    else return N2 * n1 + n2;
+  }
+  __device__ static __forceinline__ int idx_b(int k1, int k2) {
+    if constexpr (pfa) return wrap((A * k1) % N + (B * k2) % N);
+    else return k1 + N1 * k2;
+  }
+};
+
+// The twiddle of the transform's sign: conjugated for forward ones (in
+// double-float a sign change; the other types keep the product by +-1, which
+// the compiler folds).
+template <typename T, bool INV> __device__ __forceinline__ cx<T> signed_tw(cx<T> w) {
+  if constexpr (is_df<T>) {
+    if (!INV) w.y = -w.y;
+  } else {
+    w.y *= INV ? (T)1 : (T)-1;
+  }
+  return w;
+}
+
 template <typename T, int R, bool INV, int NT, int S>
 __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
   constexpr CPlan P = make_cplan(R);
@@ -116,8 +173,7 @@ __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
         if (k1 != 0) {
 #pragma unroll
           for (int q = 1; q < Rs; ++q) {
-            cx<T> w = tw[q * k1 * twstep];
-            w.y *= sg;
+            const cx<T> w = signed_tw<T, INV>(tw[q * k1 * twstep]);
             b[q] = mul<T>(b[q], w);
           }
         }
@@ -132,13 +188,36 @@ __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
 // or -1; tw[t] = exp(2 pi i t / NT), R | NT.
 template <typename T, int R, bool INV, int NT>
 __device__ __forceinline__ void dft_reg(cx<T>* x, const cx<T>* tw) {
-  constexpr RevTab rv = make_rev(R);
-  cx<T> a[R];
+  constexpr int RA = R == 12 ? 4 : R == 6 || R == 10 ? 2 : R == 15 ? 3 : 1, RB = R / RA;
+  if constexpr (is_df<T> && RA > 1) {
+    // coprime factors: no twiddles (the maps of Fac)
+    constexpr int A = RB * inv_mod(RB, RA) % R, B = RA * inv_mod(RA, RB) % R;
+    const T sg = INV ? (T)1 : (T)-1;
+    cx<T> y[R];
 #pragma unroll
-  for (int q = 0; q < R; ++q) a[q] = x[rv.v[q]];
-  reg_stages<T, R, INV, NT, 0>(a, tw);
+    for (int nb = 0; nb < RB; ++nb) {
+      cx<T> u[RA];
 #pragma unroll
-  for (int k = 0; k < R; ++k) x[k] = a[k];
+      for (int na = 0; na < RA; ++na) u[na] = x[(RB * na + RA * nb) % R];
+      dft<T, RA>(u, sg);
+#pragma unroll
+      for (int ka = 0; ka < RA; ++ka) y[ka * RB + nb] = u[ka];
+    }
+#pragma unroll
+    for (int ka = 0; ka < RA; ++ka) {
+      dft<T, RB>(y + ka * RB, sg);
+#pragma unroll
+      for (int kb = 0; kb < RB; ++kb) x[(A * ka + B * kb) % R] = y[ka * RB + kb];
+    }
+  } else {
+    constexpr RevTab rv = make_rev(R);
+    cx<T> a[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) a[q] = x[rv.v[q]];
+    reg_stages<T, R, INV, NT, 0>(a, tw);
+#pragma unroll
+    for (int k = 0; k < R; ++k) x[k] = a[k];
+  }
 }
 
 // nfft transforms of length N in shared memory (transform f at data + f
@@ -146,24 +225,24 @@ __device__ __forceinline__ void dft_reg(cx<T>* x, const cx<T>* tw) {
 // ends with __syncthreads().
 template <typename T, bool INV, int N>
 __device__ __forceinline__ void fft_nat(cx<T>* data, int nfft, int fstride, const cx<T>* tw) {
-  constexpr int N1 = fft_factor(N), N2 = N / N1;
-  static_assert(N1 > 1 && N1 <= 16 && N2 <= 16, "factor");
-  const T sg = INV ? (T)1 : (T)-1;
+  using F = Fac<T, N>;
+  constexpr int N1 = F::N1, N2 = F::N2;
   for (int t = threadIdx.x; t < nfft * N2; t += blockDim.x) {
     const int f = t / N2, n2 = t - f * N2;
     cx<T>* xf = data + f * fstride;
     cx<T> v[N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) v[n1] = xf[N2 * n1 + n2];
+    for (int n1 = 0; n1 < N1; ++n1) v[n1] = xf[F::idx_a(n1, n2)];
     dft_reg<T, N1, INV, N>(v, tw);
+    if constexpr (!F::pfa) {
 #pragma unroll
-    for (int k1 = 1; k1 < N1; ++k1) {
-      cx<T> w = tw[n2 * k1];
-      w.y *= sg;
-      v[k1] = mul<T>(v[k1], w);
+      for (int k1 = 1; k1 < N1; ++k1) {
+        const cx<T> w = signed_tw<T, INV>(tw[n2 * k1]);
+        v[k1] = mul<T>(v[k1], w);
+      }
     }
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) xf[N2 * k1 + n2] = v[k1];
+    for (int k1 = 0; k1 < N1; ++k1) xf[F::idx_a(k1, n2)] = v[k1];
   }
   __syncthreads();
   // pass 2 writes other positions than it reads: whole transforms per round,
@@ -175,16 +254,16 @@ __device__ __forceinline__ void fft_nat(cx<T>* data, int nfft, int fstride, cons
     const bool act = fl < per && f < nfft;
     cx<T> w[N2];
     if (act) {
-      const cx<T>* xf = data + f * fstride + N2 * k1;
+      const cx<T>* xf = data + f * fstride;
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[n2];
+      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[F::idx_a(k1, n2)];
       dft_reg<T, N2, INV, N>(w, tw);
     }
     __syncthreads();
     if (act) {
-      cx<T>* xf = data + f * fstride + k1;
+      cx<T>* xf = data + f * fstride;
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) xf[N1 * k2] = w[k2];
+      for (int k2 = 0; k2 < N2; ++k2) xf[F::idx_b(k1, k2)] = w[k2];
     }
   }
   __syncthreads();
@@ -246,14 +325,14 @@ __global__ void __launch_bounds__(256) ks_zinv(const double2* __restrict__ psi, 
 // threads with consecutive n2 read consecutive entries (no bank conflicts).
 template <typename T, int N, bool INV>
 __device__ __forceinline__ void fs_pass1(cx<T>* v, int n2, const cx<T>* tw, const cx<T>* tw4) {
-  constexpr int N1 = fft_factor(N), N2 = N / N1;
-  const T sg = INV ? (T)1 : (T)-1;
+  constexpr int N1 = Fac<T, N>::N1, N2 = Fac<T, N>::N2;
   dft_reg<T, N1, INV, N>(v, tw);
+  if constexpr (!Fac<T, N>::pfa) {
 #pragma unroll
-  for (int k1 = 1; k1 < N1; ++k1) {
-    cx<T> w = tw4[k1 * N2 + n2];
-    w.y *= sg;
-    v[k1] = mul<T>(v[k1], w);
+    for (int k1 = 1; k1 < N1; ++k1) {
+      const cx<T> w = signed_tw<T, INV>(tw4[k1 * N2 + n2]);
+      v[k1] = mul<T>(v[k1], w);
+    }
   }
 }
 
@@ -267,7 +346,8 @@ __device__ __forceinline__ void fs_pass1(cx<T>* v, int n2, const cx<T>* tw, cons
 template <typename T, int N, int NT, bool INV, bool FFAST, class Post>
 __device__ __forceinline__ void fs_pass2_inplace(cx<T>* data, int nf, int ld, const cx<T>* tw,
                                                  Post post) {
-  constexpr int N1 = fft_factor(N), N2 = N / N1;
+  using F = Fac<T, N>;
+  constexpr int N1 = F::N1, N2 = F::N2;
   constexpr int per = NT / N1;
   const int fl = FFAST ? (int)threadIdx.x % per : (int)threadIdx.x / N1;
   const int k1 = FFAST ? (int)threadIdx.x / per : (int)threadIdx.x - fl * N1;
@@ -276,16 +356,16 @@ __device__ __forceinline__ void fs_pass2_inplace(cx<T>* data, int nf, int ld, co
     const bool act = fl < per && k1 < N1 && f < nf;
     cx<T> w[N2];
     if (act) {
-      const cx<T>* xf = data + f * ld + N2 * k1;
+      const cx<T>* xf = data + f * ld;
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[n2];
+      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[F::idx_a(k1, n2)];
       dft_reg<T, N2, INV, N>(w, tw);
     }
     __syncthreads();
     if (act) {
-      cx<T>* xf = data + f * ld + k1;
+      cx<T>* xf = data + f * ld;
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) xf[N1 * k2] = post(f, k1 + N1 * k2, w[k2]);
+      for (int k2 = 0; k2 < N2; ++k2) xf[F::idx_b(k1, k2)] = post(f, F::idx_b(k1, k2), w[k2]);
     }
   }
   __syncthreads();
@@ -302,7 +382,8 @@ __device__ __forceinline__ void fs_pass2_inplace(cx<T>* data, int nf, int ld, co
 template <typename T, int N, int NT>
 __device__ __forceinline__ void fs_rows_mid(cx<T>* data, int nf, int ld, const cx<T>* tw,
                                             const cx<T>* tw4, const T* Vy) {
-  constexpr int N1 = fft_factor(N), N2 = N / N1;
+  using F = Fac<T, N>;
+  constexpr int N1 = F::N1, N2 = F::N2;
   constexpr int per = NT / N1;
   const int fl = (int)threadIdx.x / N1;
   const int k1 = (int)threadIdx.x - fl * N1;
@@ -311,19 +392,21 @@ __device__ __forceinline__ void fs_rows_mid(cx<T>* data, int nf, int ld, const c
     const bool act = fl < per && f < nf;
     cx<T> w[N2];
     if (act) {
-      const cx<T>* xf = data + f * ld + N2 * k1;
+      const cx<T>* xf = data + f * ld;
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[n2];
+      for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[F::idx_a(k1, n2)];
       dft_reg<T, N2, true, N>(w, tw);
-      const T* vr = Vy + (size_t)f * N + k1;
+      const T* vr = Vy + (size_t)f * N;
 #pragma unroll
-      for (int m = 0; m < N2; ++m) w[m] = scl<T>(w[m], vr[N1 * m]);
+      for (int m = 0; m < N2; ++m) w[m] = scl<T>(w[m], vr[F::idx_b(k1, m)]);
       dft_reg<T, N2, false, N>(w, tw);
+      if constexpr (!F::pfa) {
 #pragma unroll
-      for (int j = 1; j < N2; ++j) {
-        cx<T> t = tw4[k1 * N2 + j];
-        t.y = -t.y;
-        w[j] = mul<T>(w[j], t);
+        for (int j = 1; j < N2; ++j) {
+          cx<T> t = tw4[k1 * N2 + j];
+          t.y = -t.y;
+          w[j] = mul<T>(w[j], t);
+        }
       }
     }
     __syncthreads();
@@ -342,8 +425,8 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
                                                const int16_t* __restrict__ xcol_g,
                                                const T* __restrict__ V, int tw_off,
                                                const cx<T>* __restrict__ tw_g, int rows) {
-  constexpr int N1 = fft_factor(N), N2 = N / N1, LD = N + 1;
-  static_assert(N1 > 1 && N1 <= 16 && N2 <= 16, "factor");
+  using F = Fac<T, N>;
+  constexpr int N1 = F::N1, N2 = F::N2, LD = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* C = (cx<T>*)smem_raw;             // ncols x LD: columns along y
   cx<T>* R = C + (size_t)ncols * LD;       // rows x LD: rows along x
@@ -363,17 +446,17 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
   // ---- y inverse: sticks -> C
   for (int t = threadIdx.x; t < ncols * N2; t += NT) {
     const int c = t / N2, n2 = t - c * N2;
-    const int32_t* sa = stick_at + (size_t)c * N + n2;
+    const int32_t* sa = stick_at + (size_t)c * N;
     cx<T> v[N1];
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) {
-      const int st = sa[N2 * n1];
+      const int st = sa[F::idx_a(n1, n2)];
       v[n1] = st >= 0 ? plane[st] : zero;
     }
     fs_pass1<T, N, true>(v, n2, tw, tw4);
-    cx<T>* cc = C + c * LD + n2;
+    cx<T>* cc = C + c * LD;
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) cc[N2 * k1] = v[k1];
+    for (int k1 = 0; k1 < N1; ++k1) cc[F::idx_a(k1, n2)] = v[k1];
   }
   __syncthreads();
   fs_pass2_inplace<T, N, NT, true, true>(C, ncols, LD, tw, [](int, int, cx<T> v) { return v; });
@@ -387,13 +470,13 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
       cx<T> v[N1];
 #pragma unroll
       for (int n1 = 0; n1 < N1; ++n1) {
-        const int c = xcol[N2 * n1 + n2];
+        const int c = xcol[F::idx_a(n1, n2)];
         v[n1] = c >= 0 ? C[c * LD + y0 + r] : zero;
       }
       fs_pass1<T, N, true>(v, n2, tw, tw4);
-      cx<T>* rr = R + r * LD + n2;
+      cx<T>* rr = R + r * LD;
 #pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) rr[N2 * k1] = v[k1];
+      for (int k1 = 0; k1 < N1; ++k1) rr[F::idx_a(k1, n2)] = v[k1];
     }
     __syncthreads();
     fs_rows_mid<T, N, NT>(R, nr, LD, tw, tw4, Vz + (size_t)y0 * N);
@@ -407,7 +490,8 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
       dft_reg<T, N1, false, N>(v, tw);
 #pragma unroll
       for (int l = 0; l < N1; ++l) {
-        const int c = xcol[j + N2 * l];
+        // four-step: output j + N2 l; coprime: the input map as output map
+        const int c = xcol[F::pfa ? F::idx_a(l, j) : j + N2 * l];
         if (c >= 0) C[c * LD + y0 + r] = v[l];
       }
     }
@@ -417,30 +501,36 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
   // ---- y forward: C -> sticks
   for (int t = threadIdx.x; t < ncols * N2; t += NT) {
     const int c = t / N2, n2 = t - c * N2;
-    cx<T>* cc = C + c * LD + n2;
+    cx<T>* cc = C + c * LD;
     cx<T> v[N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) v[n1] = cc[N2 * n1];
+    for (int n1 = 0; n1 < N1; ++n1) v[n1] = cc[F::idx_a(n1, n2)];
     fs_pass1<T, N, false>(v, n2, tw, tw4);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) cc[N2 * k1] = v[k1];
+    for (int k1 = 0; k1 < N1; ++k1) cc[F::idx_a(k1, n2)] = v[k1];
   }
   __syncthreads();
   for (int t = threadIdx.x; t < ncols * N1; t += NT) {
     const int c = t / N1, k1 = t - c * N1;
-    const cx<T>* cc = C + c * LD + N2 * k1;
+    const cx<T>* cc = C + c * LD;
     cx<T> w[N2];
 #pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) w[n2] = cc[n2];
+    for (int n2 = 0; n2 < N2; ++n2) w[n2] = cc[F::idx_a(k1, n2)];
     dft_reg<T, N2, false, N>(w, tw);
-    const int32_t* sa = stick_at + (size_t)c * N + k1;
+    const int32_t* sa = stick_at + (size_t)c * N;
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) {
-      const int st = sa[N1 * k2];
+      const int st = sa[F::idx_b(k1, k2)];
       if (st >= 0) plane[st] = w[k2];
     }
   }
 }
+
+// Threads of a plane block.  Double-float threads hold 128 registers: two blocks
+// of 256 an SM, whose barriers then overlap with the other's arithmetic (90^3,
+// 128 bands: 2.92 ms, against 3.45 ms in one block of 512 and 3.90 in one of
+// 384).
+template <typename T> constexpr int plane_threads = std::is_same<T, float>::value ? 512 : 256;
 
 // Shared memory of the plane pass for `rows` rows per chunk.
 template <typename T, int N> constexpr size_t ks_plane_smem(int ncols, int rows) {
@@ -518,6 +608,7 @@ template <typename T, int N> int plane_rows_heuristic(int ncols) {
 }
 
 template <typename T, int N> int plane_rows(System& s, const PassArgs& a) {
+  constexpr int NT = plane_threads<T>;
   static std::mutex mu;
   static std::map<int, int> chosen;  // ncols -> rows
   std::lock_guard<std::mutex> lock(mu);
@@ -550,7 +641,7 @@ template <typename T, int N> int plane_rows(System& s, const PassArgs& a) {
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {
         if (rep == 1) PWH_CUDA(cudaEventRecord(e0, a.st));
-        ks_plane<T, N, 512><<<dim3(N, a.bb), 512, smem, a.st>>>(
+        ks_plane<T, N, NT><<<dim3(N, a.bb), NT, smem, a.st>>>(
             Wt, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V,
             s.plan[0].tw_off, (const cx<T>*)a.tw, r);
         PWH_LAUNCH_CHECK();
@@ -574,7 +665,7 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
   static std::once_flag once;
   std::call_once(once, [] {
     cudaFuncSetAttribute(ks_zinv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(ks_plane<T, N, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(ks_plane<T, N, plane_threads<T>>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaFuncSetAttribute(ks_zfwd<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   });
   const cx<T>* tw = (const cx<T>*)a.tw;
@@ -587,8 +678,9 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
                                                  s.d_perm, W, a.wband, a.spb);
       break;
     case SPEC_PLANE: {
+      constexpr int NT = plane_threads<T>;
       const int rows = plane_rows<T, N>(s, a);
-      ks_plane<T, N, 512><<<dim3(N, a.bb), 512, ks_plane_smem<T, N>(s.ncols, rows), a.st>>>(
+      ks_plane<T, N, NT><<<dim3(N, a.bb), NT, ks_plane_smem<T, N>(s.ncols, rows), a.st>>>(
           W, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V, s.plan[0].tw_off,
           tw, rows);
       break;
