@@ -13,6 +13,7 @@
 // workspace and summed by k_splitk_reduce in a fixed order (deterministic).
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include "common.cuh"
 #include "gemm.cuh"
@@ -25,6 +26,8 @@ namespace pwh {
 // complex outputs per thread (thread (tx, ty) owns rows tx + (BM/TM) i and
 // columns ty + (BN/TN) j), K-slabs of BK: the next slab is fetched into
 // registers while the current one is multiplied out of shared memory.
+template <int V> using I = std::integral_constant<int, V>;
+
 template <typename TS, typename T, bool CONJ_A, int BM, int BN, int TM, int TN, int BK>
 __global__ void __launch_bounds__(256) k_cgemm(int M, int N, int K, const cx<TS>* __restrict__ A,
                                                int64_t lda, const cx<TS>* __restrict__ B,
@@ -201,19 +204,20 @@ __global__ void __launch_bounds__(256) k_splitk_reduce_wide(int M, int N, int ns
 // Tile shapes (BM, BN, TM, TN, BK) by the width N of the product: narrow
 // products (a few unconverged bands) take tall thin tiles so that no
 // arithmetic is spent on padding columns; FP32 takes 8 x 8 (or 8 x 4)
-// outputs per thread, FP64 4 x 4 (its pipe, not shared memory, is the limit).
+// outputs per thread, FP64 by plan64 (its pipe, not shared memory, is the
+// limit).
 template <typename TS, typename T, int BM, int BN, int TM, int TN, int BK>
 static void cgemm_launch(System& s, bool conjA, int M, int N, int K, cx<TS> alpha, const cx<TS>* A,
                          int64_t lda, const cx<TS>* B, int64_t ldb, cx<TS> beta, cx<TS>* C,
-                         int64_t ldc, cudaStream_t st, const double* rowscale) {
+                         int64_t ldc, cudaStream_t st, const double* rowscale, int split = 0) {
   const int gm = (M + BM - 1) / BM, gn = (N + BN - 1) / BN;
   const int tiles = gm * gn;
   // split the reduction when the output tiles alone fill less than one wave
   // (into about two blocks per SM, chunks of at least 32: small square
   // products such as the eigensolver's n x n x n ones still spread out)
   // (the partials of a split stay below 64 MB)
-  int nsplit = 1;
-  if (tiles < 152 && K > 2 * BK) {
+  int nsplit = std::max(1, split);  // split > 0: the caller's choice
+  if (split == 0 && tiles < 152 && K > 2 * BK) {
     nsplit = std::min((2 * 152 + tiles - 1) / tiles, std::max(1, K / 32));
     const int64_t cap = std::max<int64_t>(1, ((int64_t)64 << 20) / ((int64_t)M * N * (int64_t)sizeof(cx<TS>)));
     nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(nsplit, cap));
@@ -254,6 +258,39 @@ static void cgemm_launch(System& s, bool conjA, int M, int N, int K, cx<TS> alph
   }
 }
 
+// Tile and split-K of an FP64 product on the FP64 pipe: the least modelled
+// clocks, waves of blocks over 152 SMs times a block's multiply-adds (four a
+// complex pair at the measured 1.6 a clock of an SM) and 1,200 clocks of latency,
+// plus the reduction of the partials.  A tile much larger than the product
+// computes padding, and few tiles leave the pipe of most SMs idle: 32 x 16 over
+// K = 1503 took 176 us in 256 x 16 tiles and takes 20, 1503 x 16 over K = 32 139 us
+// on six of them and takes 14, 256^3 143 us and takes 45 (oz_gemm).
+struct Plan64 {
+  int shape, split;
+  double us;  // modelled time
+};
+constexpr int kShape64[7][2] = {{64, 64}, {128, 32}, {256, 16}, {256, 8}, {32, 32}, {32, 16}, {16, 16}};
+static Plan64 plan64(int M, int N, int K, bool part) {
+  Plan64 best{0, 1, 1e300};
+  for (int i = 0; i < 7; ++i) {
+    const int BM = kShape64[i][0], BN = kShape64[i][1];
+    const int64_t tiles = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    for (int w = 0; w <= 6; ++w) {
+      int split = w == 0 ? 1 : (int)((152 * (int64_t)w + tiles - 1) / tiles);
+      split = std::max(1, std::min(split, std::min(256, K / 16)));
+      if ((double)split * M * N * 16.0 > 64.0 * (1 << 20)) continue;
+      const int chunk = (((K + split - 1) / split) + 15) / 16 * 16;
+      split = std::max(1, (K + chunk - 1) / std::max(chunk, 1));
+      const double waves = (double)((tiles * split + 151) / 152);
+      double clk = waves * (2.5 * BM * BN * chunk + 1200.0);
+      if (split > 1 || part) clk += 5000.0 + split * (double)M * N * 32.0 / 3000.0;
+      if (clk < best.us) best = {i, split, clk};
+    }
+  }
+  best.us /= 2000.0;  // 2 GHz
+  return best;
+}
+
 template <typename TS, typename T>
 static void cgemm_impl(System& s, bool conjA, int M, int N, int K, cx<TS> alpha, const cx<TS>* A,
                        int64_t lda, const cx<TS>* B, int64_t ldb, cx<TS> beta, cx<TS>* C,
@@ -273,19 +310,35 @@ static void cgemm_impl(System& s, bool conjA, int M, int N, int K, cx<TS> alpha,
     else
       cgemm_launch<TS, T, 256, 16, 8, 2, 8>(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
   } else {
-    if (N > 32)
-      cgemm_launch<TS, T, 64, 64, 4, 4, 16>(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
-    else if (N > 16)
-      cgemm_launch<TS, T, 128, 32, 4, 4, 16>(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
-    else if (N > 8)
-      cgemm_launch<TS, T, 256, 16, 4, 4, 8>(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
-    else
-      cgemm_launch<TS, T, 256, 8, 4, 2, 8>(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
+    const Plan64 p = plan64(M, N, K, rowscale != nullptr);
+    auto run = [&](auto bm, auto bn, auto tm, auto tn, auto bk) {
+      cgemm_launch<TS, T, decltype(bm)::value, decltype(bn)::value, decltype(tm)::value,
+                   decltype(tn)::value, decltype(bk)::value>(s, conjA, M, N, K, alpha, A, lda, B, ldb,
+                                                             beta, C, ldc, st, rowscale, p.split);
+    };
+    switch (p.shape) {
+      case 0: run(I<64>{}, I<64>{}, I<4>{}, I<4>{}, I<16>{}); break;
+      case 1: run(I<128>{}, I<32>{}, I<4>{}, I<4>{}, I<16>{}); break;
+      case 2: run(I<256>{}, I<16>{}, I<4>{}, I<4>{}, I<8>{}); break;
+      case 3: run(I<256>{}, I<8>{}, I<4>{}, I<2>{}, I<8>{}); break;
+      case 4: run(I<32>{}, I<32>{}, I<2>{}, I<2>{}, I<16>{}); break;
+      case 5: run(I<32>{}, I<16>{}, I<2>{}, I<1>{}, I<16>{}); break;
+      default: run(I<16>{}, I<16>{}, I<1>{}, I<1>{}, I<16>{}); break;
+    }
   }
 }
 
-// FP64 products of at least kOzMinFlops go to the tensor cores as integer
-// products by residues (oz_gemm).
+// Whether an FP64 product goes to the tensor cores (oz_gemm): at least
+// kOzMinFlops, and the modelled time there is the smaller: about 40 us of launches
+// and latency, the operands read twice and written as 64 bytes a complex number
+// (5 TB/s), 128 tensor operations a complex multiply-add (1.2 PFLOP/s).  Products
+// of a few columns stay on the FP64 pipe whatever their length.
+static bool oz_wins(int M, int N, int K) {
+  if (8.0 * M * (double)N * K < kOzMinFlops) return false;
+  const double oz = 40.0 + ((double)M + N) * K * 96.0 / 5e6 + 128.0 * M * (double)N * K / 1.2e9 +
+                    (double)M * N * 80.0 / 3e6;
+  return oz < plan64(M, N, K, false).us;
+}
 
 // The sliced tensor-core paths launch one block row per column of A (A^H B)
 // and of B along grid y, and K / 64 blocks along grid y of the A B slicing:
@@ -314,8 +367,7 @@ void cgemm(System& s, bool conjA, int M, int N, int K, cx<T> alpha, const cx<T>*
            const cx<T>* B, int64_t ldb, cx<T> beta, cx<T>* C, int64_t ldc, cudaStream_t st,
            const double* rowscale) {
   if constexpr (sizeof(T) == 8) {
-    if (K > 0 && 8.0 * M * (double)N * K >= kOzMinFlops &&
-        slice_grid_ok(conjA, M, N, K)) {
+    if (K > 0 && oz_wins(M, N, K) && slice_grid_ok(conjA, M, N, K)) {
       oz_gemm(s, conjA, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st, rowscale);
       return;
     }
