@@ -196,6 +196,7 @@ struct System {
 
   // device: maps and tables
   int32_t* d_int_to_pub = nullptr;
+  int32_t* d_pub_to_int = nullptr;  // its inverse
   double* d_kin = nullptr;          // internal order
   int32_t* d_stick_off = nullptr;
   int32_t* d_stick_of = nullptr;    // stick of each internal plane wave
@@ -217,7 +218,7 @@ struct System {
   bool have_v = false;
   double vbar = 0.0;                // mean of V_LOC(r) over the grid
   double* d_v64 = nullptr;
-  float* d_v32 = nullptr;
+  float* d_v32 = nullptr;          // V in FP32: [i3][i1][i2] where the box has compiled passes
   float2* d_vdf = nullptr;          // V as double-float pairs (hi, lo)
 
   // projectors (internal plane-wave order, column-major ld = npw)

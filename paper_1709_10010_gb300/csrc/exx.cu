@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "dense.cuh"
+#include "fft_axis64.cuh"
 #include "gemm.cuh"
 
 namespace pwh {
@@ -194,6 +195,33 @@ struct ExxScratch {
   }
 };
 
+// pair[j] <- the potentials v_j of the pair densities conj(U_j) P, jb boxes.  With
+// compiled edges the pair density is formed as the first axis is loaded, and the
+// last forward axis, the Coulomb factor and the first inverse axis are one kernel:
+// five passes over the pair boxes instead of eight.
+static void pair_potentials(System& s, const double2* Uj, const double2* P, double2* pair,
+                            int64_t nbox, int jb) {
+  if (axis64_planes(s)) {
+    AxisArgs a{pair, nbox, jb, 2, Uj, P, s.d_kern};
+    axis64_box(s, AX_PAIR, a);
+    a.axis = 1;
+    axis64_box(s, AX_FWD, a);
+    a.axis = 0;
+    axis64_box(s, AX_KERN, a);
+    a.axis = 1;
+    axis64_box(s, AX_INV, a);
+    a.axis = 2;
+    axis64_box(s, AX_INV, a);
+    return;
+  }
+  k_exx_pair<<<exx_grid(nbox * jb), 256, 0, s.stream>>>(Uj, P, pair, nbox, jb);
+  PWH_LAUNCH_CHECK();
+  box_fft(s, pair, false, jb, nbox);
+  k_exx_coulomb<<<exx_grid(nbox * jb), 256, 0, s.stream>>>(pair, s.d_kern, nbox, jb);
+  PWH_LAUNCH_CHECK();
+  box_fft(s, pair, true, jb, nbox);
+}
+
 // out[:, i] = V_x phi_i for nb bands (public order, device), occupied bands
 // psi_occ (public order, device) with host weights occ.
 static void exx_apply(System& s, int nocc, const double2* psi_occ, int64_t ld_occ,
@@ -228,12 +256,7 @@ static void exx_apply(System& s, int nocc, const double2* psi_occ, int64_t ld_oc
     for (int j0 = 0; j0 < nocc; j0 += J) {
       const int jb = std::min(J, nocc - j0);
       const double2* Uj = U + (size_t)j0 * nbox;
-      k_exx_pair<<<exx_grid(nbox * jb), 256, 0, st>>>(Uj, P, pair, nbox, jb);
-      PWH_LAUNCH_CHECK();
-      box_fft(s, pair, false, jb, nbox);
-      k_exx_coulomb<<<exx_grid(nbox * jb), 256, 0, st>>>(pair, s.d_kern, nbox, jb);
-      PWH_LAUNCH_CHECK();
-      box_fft(s, pair, true, jb, nbox);
+      pair_potentials(s, Uj, P, pair, nbox, jb);
       k_exx_acc<<<exx_grid(nbox), 256, 0, st>>>(Uj, pair, f + j0, W, nbox, jb);
       PWH_LAUNCH_CHECK();
     }
@@ -271,12 +294,7 @@ static void exx_apply_self(System& s, int nocc, const double2* psi, int64_t ld, 
     for (int j0 = 0; j0 <= i; j0 += J) {
       const int jb = std::min(J, i + 1 - j0);
       const double2* Uj = U + (size_t)j0 * nbox;
-      k_exx_pair<<<exx_grid(nbox * jb), 256, 0, st>>>(Uj, Ui, pair, nbox, jb);
-      PWH_LAUNCH_CHECK();
-      box_fft(s, pair, false, jb, nbox);
-      k_exx_coulomb<<<exx_grid(nbox * jb), 256, 0, st>>>(pair, s.d_kern, nbox, jb);
-      PWH_LAUNCH_CHECK();
-      box_fft(s, pair, true, jb, nbox);
+      pair_potentials(s, Uj, Ui, pair, nbox, jb);
       // band i: sources j0.. (v_ij); bands j0.. (j < i): source i (conj v_ij)
       k_exx_acc<<<exx_grid(nbox), 256, 0, st>>>(Uj, pair, f + j0, Wi, nbox, jb);
       PWH_LAUNCH_CHECK();

@@ -33,6 +33,7 @@
 
 #include "common.cuh"
 #include "df.cuh"
+#include "fft_axis64.cuh"
 #include "fft_device.cuh"
 #include "fft_spec.cuh"
 
@@ -130,6 +131,10 @@ __device__ void fft_block(cx<T>* data, int nfft, int fstride, int estride, const
     __syncthreads();
   }
 }
+
+// FP64 has no compiled cubic passes of its own (double-float, or the axis-wise
+// transforms)
+template <> bool spec_pass<double>(SpecPass, System&, const PassArgs&) { return false; }
 
 template <typename T> struct TwT;
 template <> struct TwT<double> { static const double2* get(const System& s) { return s.d_tw64; } };
@@ -302,6 +307,52 @@ static size_t plane_smem(const System& s, int rows) {
          (size_t)(s.n1 + s.n2) * sizeof(int16_t);
 }
 
+// Bands whose sticks and columns of the axis-wise passes fit about 64 MB.
+static int axes_batch(const System& s, int nb) {
+  const int64_t per = ((int64_t)s.nsticks + (int64_t)s.ncols * s.n2) * s.n3 * (int64_t)sizeof(double2);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nb, 65535), (64ll << 20) / per));
+}
+
+// The FP64 local part on a box whose three edges have compiled axis transforms
+// (boxes that are not cubic, cubic ones without double-float passes): z inverse,
+// y inverse, x inverse times V x forward, y forward, z forward, each its own
+// kernel over blocks of 16 lines, the columns between them in L2.  Against the
+// plane kernel of the runtime plans, 61 bands on a 60 x 60 x 90 box: planes 2.98 ->
+// 2.13 ms, z passes 0.34 -> 0.33.  The density of 128 bands on 90^3: 11.4 -> 7.5 ms.
+static void local_kinetic_axes(System& s, int nb, const double2* psi, int64_t ldp, double2* hpsi,
+                               int64_t ldh, cudaStream_t st, const float2* vnl, int64_t ldv) {
+  const int64_t wband = (int64_t)s.n3 * s.nsticks, cband = (int64_t)s.n3 * s.ncols * s.n2;
+  const int batch = axes_batch(s, nb);
+  ensure(s.ws_fft, (size_t)batch * (wband + cband) * sizeof(double2));
+  double2* W = (double2*)s.ws_fft.p;
+  const int spb = stick_block(s.n3);
+  const size_t zsmem = ((size_t)spb * (s.n3 + 1) + s.n3) * sizeof(double2) + s.n3 * sizeof(int16_t);
+  auto l2 = [](int n) { return std::log2((double)n); };
+  const double fz = 5.0 * s.n3 * l2(s.n3) * s.nsticks, bw = 16.0 * (double)wband;
+  const double fp = 2.0 * s.n3 * (s.ncols * 5.0 * s.n2 * l2(s.n2) + s.n2 * 5.0 * s.n1 * l2(s.n1));
+  for (int b0 = 0; b0 < nb; b0 += batch) {
+    const int bb = std::min(batch, nb - b0);
+    const float2* vb = vnl ? vnl + (size_t)b0 * ldv : nullptr;
+    const PassArgs za{psi + (size_t)b0 * ldp, ldp, hpsi + (size_t)b0 * ldh, ldh, W, wband, spb,
+                      zsmem, 0, 0, bb, nullptr, nullptr, st, vb, ldv};
+    const PlaneArgs pa{W, wband, W + (size_t)batch * wband, bb, s.d_v64, nullptr, 0, nullptr};
+    {
+      TimedScope ts(s, KF_FFT_ZINV64, st, bb * fz, bb * (16.0 * s.npw + bw));
+      axis64_z(s, true, za);
+    }
+    {
+      TimedScope ts(s, KF_FFT_PLANE64, st, bb * fp, bb * 2.0 * bw + 8.0 * s.n1 * s.n2 * s.n3);
+      axis64_plane(s, PL_YINV, pa);
+      axis64_plane(s, PL_XV, pa);
+      axis64_plane(s, PL_YFWD, pa);
+    }
+    {
+      TimedScope ts(s, KF_FFT_ZFWD64, st, bb * fz, bb * (bw + 40.0 * s.npw));
+      axis64_z(s, false, za);
+    }
+  }
+}
+
 template <typename T>
 void local_kinetic(System& s, int nb, const double2* psi, int64_t ldp, double2* hpsi, int64_t ldh,
                    cudaStream_t st, const float2* vnl, int64_t ldv) {
@@ -313,6 +364,10 @@ void local_kinetic(System& s, int nb, const double2* psi, int64_t ldp, double2* 
     // about 2^-46 an operation)
     if (spec_box(s)) {
       local_kinetic<df>(s, nb, psi, ldp, hpsi, ldh, st, vnl, ldv);
+      return;
+    }
+    if (axis64_planes(s)) {
+      local_kinetic_axes(s, nb, psi, ldp, hpsi, ldh, st, vnl, ldv);
       return;
     }
   }
@@ -528,6 +583,28 @@ __global__ void __launch_bounds__(256) k_box_fft_axis(double2* __restrict__ box,
 void density_accumulate(System& s, int nb, const double2* psi_int, const double* occ_dev,
                         double* rho_int) {
   using T = double;
+  if (axis64_planes(s)) {
+    const int64_t wb = (int64_t)s.n3 * s.nsticks, cb = (int64_t)s.n3 * s.ncols * s.n2;
+    const int batch = axes_batch(s, nb);
+    ensure(s.ws_fft, (size_t)batch * (wb + cb) * sizeof(double2));
+    double2* W = (double2*)s.ws_fft.p;
+    const int spb = stick_block(s.n3);
+    const size_t zsmem = ((size_t)spb * (s.n3 + 1) + s.n3) * sizeof(double2) + s.n3 * sizeof(int16_t);
+    for (int b0 = 0; b0 < nb; b0 += batch) {
+      const int bb = std::min(batch, nb - b0);
+      const PassArgs za{psi_int + (size_t)b0 * s.npw, s.npw, nullptr, 0, W, wb, spb, zsmem, 0, 0,
+                        bb, nullptr, nullptr, s.stream, nullptr, 0};
+      axis64_z(s, true, za);
+      // slices of bands: about four waves of row groups over the GPU
+      const int rowgroups = ((s.n2 + 15) / 16) * s.n3;
+      const int slices = std::max(1, std::min(bb, (8 * 4 * 152 + rowgroups - 1) / rowgroups));
+      const PlaneArgs pa{W, wb, W + (size_t)batch * wb, bb, nullptr, occ_dev + b0,
+                         (bb + slices - 1) / slices, rho_int};
+      axis64_plane(s, PL_YINV, pa);
+      axis64_plane(s, PL_XDENS, pa);
+    }
+    return;
+  }
   const int64_t wband = (int64_t)s.n3 * s.nsticks;
   const int64_t per = wband * (int64_t)sizeof(cx<T>);
   const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(nb, (64ll << 20) / std::max<int64_t>(per, 1)));
@@ -569,6 +646,15 @@ void box_fft(System& s, double2* box, bool inverse, int nbox, int64_t bstride) {
     cudaFuncSetAttribute(k_box_fft_axis, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   });
   for (int axis = 2; axis >= 0; --axis) {
+    if (axis64_size(n[axis])) {
+      AxisArgs a{};
+      a.box = box;
+      a.bstride = bstride;
+      a.nbox = nbox;
+      a.axis = axis;
+      axis64_box(s, inverse ? AX_INV : AX_FWD, a);
+      continue;
+    }
     const FftPlan& pl = s.plan[axis];
     const int64_t nlines = (int64_t)n[0] * n[1] * n[2] / n[axis];
     // lines a block: 16 (a 256-byte run of the fast axis), fewer if n is large

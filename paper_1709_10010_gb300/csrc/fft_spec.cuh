@@ -1,6 +1,6 @@
 // FFT passes specialised at compile time for cubic boxes of common sizes
 // (interface).  The kernels are in fft_spec_impl.cuh, instantiated once per
-// arithmetic in fft_spec32.cu, fft_spec64.cu and fft_specdf.cu (double-float).
+// arithmetic in fft_spec32.cu and fft_specdf.cu (double-float).
 #pragma once
 #include "common.cuh"
 

@@ -100,10 +100,12 @@ constexpr int fft_factor(int n) {
   return best;
 }
 
-// Whether T is double-float: its arithmetic is the passes' limit, so it takes
-// the factorisation with the fewest products.  The other types keep theirs.
+// Whether the arithmetic of T is the passes' limit (double-float on the FP32
+// pipes, FP64 on its own): then the factorisation with the fewest products.
+// FP32 is bound by shared memory and keeps the four-step one.
 struct df;
 template <typename T> constexpr bool is_df = std::is_same<T, df>::value;
+template <typename T> constexpr bool few_products = is_df<T> || std::is_same<T, double>::value;
 
 constexpr int gcd_of(int a, int b) { return b ? gcd_of(b, a % b) : a; }
 constexpr int inv_mod(int a, int m) {
@@ -128,7 +130,7 @@ constexpr int coprime_factor(int n) {
 // idx_b(k1, k2) the output.  Forward transforms of the rows run with the two
 // maps exchanged.
 template <typename T, int N> struct Fac {
-  static constexpr bool pfa = is_df<T> && coprime_factor(N) > 1;
+  static constexpr bool pfa = few_products<T> && coprime_factor(N) > 1;
   static constexpr int N1 = pfa ? coprime_factor(N) : fft_factor(N), N2 = N / N1;
   static_assert(N1 > 1 && N1 <= 16 && N2 <= 16, "factor");
   static constexpr int A = pfa ? N2 * inv_mod(N2, N1) % N : 1;
@@ -189,7 +191,7 @@ __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
 template <typename T, int R, bool INV, int NT>
 __device__ __forceinline__ void dft_reg(cx<T>* x, const cx<T>* tw) {
   constexpr int RA = R == 12 ? 4 : R == 6 || R == 10 ? 2 : R == 15 ? 3 : 1, RB = R / RA;
-  if constexpr (is_df<T> && RA > 1) {
+  if constexpr (few_products<T> && RA > 1) {
     // coprime factors: no twiddles (the maps of Fac)
     constexpr int A = RB * inv_mod(RB, RA) % R, B = RA * inv_mod(RA, RB) % R;
     const T sg = INV ? (T)1 : (T)-1;
@@ -419,6 +421,40 @@ __device__ __forceinline__ void fs_rows_mid(cx<T>* data, int nf, int ld, const c
   __syncthreads();
 }
 
+// The same for FP32, which shared memory bounds: neighbouring threads take
+// neighbouring rows (odd ld: no bank conflicts, the twiddle of a warp one or two
+// words), V from its [z][x][y] copy (coalesced along the rows), and slot (k1, n2) at
+// k1 + N1 n2, which for fixed k1 are both the thread's inputs and its outputs: no
+// barrier between its loads and its stores.  The whole plane pass at 144^3, 512
+// bands: 10.85 -> 8.28 ms, at 90^3, 128 bands: 0.541 -> 0.461 (shared memory pipe 75%
+// busy, issue slots 67%).
+template <int N, int NT>
+__device__ __forceinline__ void fs_rows_mid32(float2* data, int nf, int ld, const float2* tw,
+                                              const float2* tw4, const float* Vt) {
+  constexpr int N1 = Fac<float, N>::N1, N2 = Fac<float, N>::N2;
+  for (int t = threadIdx.x; t < nf * N1; t += NT) {
+    const int k1 = t / nf, f = t - k1 * nf;
+    float2* xf = data + f * ld + k1;
+    float2 w[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) w[n2] = xf[N1 * n2];
+    dft_reg<float, N2, true, N>(w, tw);
+    const float* vr = Vt + (size_t)k1 * N + f;
+#pragma unroll
+    for (int m = 0; m < N2; ++m) w[m] = scl<float>(w[m], vr[(size_t)N1 * N * m]);
+    dft_reg<float, N2, false, N>(w, tw);
+#pragma unroll
+    for (int j = 1; j < N2; ++j) {
+      float2 c = tw4[k1 * N2 + j];
+      c.y = -c.y;
+      w[j] = mul<float>(w[j], c);
+    }
+#pragma unroll
+    for (int j = 0; j < N2; ++j) xf[N1 * j] = w[j];
+  }
+  __syncthreads();
+}
+
 template <typename T, int N, int NT>
 __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wband, int nsticks,
                                                int ncols, const int32_t* __restrict__ stick_at,
@@ -427,6 +463,7 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
                                                const cx<T>* __restrict__ tw_g, int rows) {
   using F = Fac<T, N>;
   constexpr int N1 = F::N1, N2 = F::N2, LD = N + 1;
+  constexpr bool RF = std::is_same<T, float>::value;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* C = (cx<T>*)smem_raw;             // ncols x LD: columns along y
   cx<T>* R = C + (size_t)ncols * LD;       // rows x LD: rows along x
@@ -466,7 +503,9 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
   for (int y0 = 0; y0 < N; y0 += rows) {
     const int nr = min(rows, N - y0);
     for (int t = threadIdx.x; t < nr * N2; t += NT) {
-      const int r = t / N2, n2 = t - r * N2;
+      // FP32: neighbouring threads on neighbouring rows, the column of x and the
+      // twiddles one word a warp (fs_rows_mid32)
+      const int r = RF ? t % nr : t / N2, n2 = RF ? t / nr : t - r * N2;
       cx<T> v[N1];
 #pragma unroll
       for (int n1 = 0; n1 < N1; ++n1) {
@@ -476,10 +515,13 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
       fs_pass1<T, N, true>(v, n2, tw, tw4);
       cx<T>* rr = R + r * LD;
 #pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) rr[F::idx_a(k1, n2)] = v[k1];
+      for (int k1 = 0; k1 < N1; ++k1) rr[RF ? k1 + N1 * n2 : F::idx_a(k1, n2)] = v[k1];
     }
     __syncthreads();
-    fs_rows_mid<T, N, NT>(R, nr, LD, tw, tw4, Vz + (size_t)y0 * N);
+    if constexpr (RF)
+      fs_rows_mid32<N, NT>(R, nr, LD, tw, tw4, Vz + y0);
+    else
+      fs_rows_mid<T, N, NT>(R, nr, LD, tw, tw4, Vz + (size_t)y0 * N);
     // forward pass 2 (N1-point DFTs over k1): X[j + N2 l], only the columns
     for (int t = threadIdx.x; t < nr * N2; t += NT) {
       const int r = t % nr, j = t / nr;  // neighbouring rows: conflict-free
@@ -500,7 +542,7 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
 
   // ---- y forward: C -> sticks
   for (int t = threadIdx.x; t < ncols * N2; t += NT) {
-    const int c = t / N2, n2 = t - c * N2;
+    const int c = RF ? t % ncols : t / N2, n2 = RF ? t / ncols : t - c * N2;
     cx<T>* cc = C + c * LD;
     cx<T> v[N1];
 #pragma unroll
@@ -529,8 +571,11 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
 // Threads of a plane block.  Double-float threads hold 128 registers: two blocks
 // of 256 an SM, whose barriers then overlap with the other's arithmetic (90^3,
 // 128 bands: 2.92 ms, against 3.45 ms in one block of 512 and 3.90 in one of
-// 384).
-template <typename T> constexpr int plane_threads = std::is_same<T, float>::value ? 512 : 256;
+// 384).  FP32 waits for shared memory: 256 threads, two blocks an SM by shared
+// memory, at 90^3 (0.461 ms for 128 bands, 0.470 with 512); one block of 1,024 where
+// the columns leave room for one (144^3, 512 bands: 8.28 ms, 8.43 with 512, 9.8 with
+// 768).
+template <typename T, int N> constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 120 ? 1024 : 256) : 256;
 
 // Shared memory of the plane pass for `rows` rows per chunk.
 template <typename T, int N> constexpr size_t ks_plane_smem(int ncols, int rows) {
@@ -608,7 +653,7 @@ template <typename T, int N> int plane_rows_heuristic(int ncols) {
 }
 
 template <typename T, int N> int plane_rows(System& s, const PassArgs& a) {
-  constexpr int NT = plane_threads<T>;
+  constexpr int NT = plane_threads<T, N>;
   static std::mutex mu;
   static std::map<int, int> chosen;  // ncols -> rows
   std::lock_guard<std::mutex> lock(mu);
@@ -665,7 +710,7 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
   static std::once_flag once;
   std::call_once(once, [] {
     cudaFuncSetAttribute(ks_zinv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(ks_plane<T, N, plane_threads<T>>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(ks_plane<T, N, plane_threads<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaFuncSetAttribute(ks_zfwd<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   });
   const cx<T>* tw = (const cx<T>*)a.tw;
@@ -678,7 +723,7 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
                                                  s.d_perm, W, a.wband, a.spb);
       break;
     case SPEC_PLANE: {
-      constexpr int NT = plane_threads<T>;
+      constexpr int NT = plane_threads<T, N>;
       const int rows = plane_rows<T, N>(s, a);
       ks_plane<T, N, NT><<<dim3(N, a.bb), NT, ks_plane_smem<T, N>(s.ncols, rows), a.st>>>(
           W, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V, s.plan[0].tw_off,

@@ -16,6 +16,7 @@
 #include <numeric>
 
 #include "common.cuh"
+#include "fft_spec.cuh"
 
 namespace pwh {
 
@@ -84,7 +85,7 @@ KernelTimer::~KernelTimer() {
 System::~System() {
   if (stream) cudaStreamSynchronize(stream);
   free_davidson_ws(dav);
-  void* ptrs[] = {d_int_to_pub, d_kin, d_stick_off, d_stick_of, d_zpos, d_stick_col,
+  void* ptrs[] = {d_int_to_pub, d_pub_to_int, d_kin, d_stick_off, d_stick_of, d_zpos, d_stick_col,
                   d_stick_y, d_col_x, d_stick_at, d_xcol, d_tw64, d_tw32, d_twdf, d_perm, d_v64, d_v32, d_vdf, d_beta64,
                   d_ddiag, d_dfull, d_beta32, d_beta_bf16, d_beta_bf16_t,
                   ws_fft.p, ws_vnl.p, ws_grid.p, ws_tune.p, ws_psi.p, ws_hpsi.p, ws_becp.p, ws_split.p, ws_host.p,
@@ -238,6 +239,9 @@ template <typename T> static T* upload(const std::vector<T>& v, cudaStream_t st)
 static void upload_basis(System& s) {
   cudaStream_t st = s.stream;
   s.d_int_to_pub = upload(s.int_to_pub, st);
+  std::vector<int32_t> pub_to_int(s.npw);
+  for (int64_t i = 0; i < s.npw; ++i) pub_to_int[s.int_to_pub[i]] = (int32_t)i;
+  s.d_pub_to_int = upload(pub_to_int, st);
   std::vector<double> kin(s.npw);
   std::vector<int32_t> stick_of(s.npw);
   std::vector<int16_t> zpos(s.npw);
@@ -271,7 +275,7 @@ static void upload_basis(System& s) {
 
 // ------------------------------------------------------- device helpers -----
 __global__ void k_potential_layout(const double* __restrict__ v, int n1, int n2, int n3,
-                                   double scale, double* __restrict__ v64,
+                                   double scale, int v32_xy, double* __restrict__ v64,
                                    float* __restrict__ v32, float2* __restrict__ vdf) {
   int64_t tot = (int64_t)n1 * n2 * n3;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot;
@@ -283,7 +287,8 @@ __global__ void k_potential_layout(const double* __restrict__ v, int n1, int n2,
     int i3 = (int)(r / n2);
     double x = v[((int64_t)i1 * n2 + i2) * n3 + i3] * scale;
     v64[t] = x;
-    v32[t] = (float)x;
+    // the compiled FP32 plane passes read neighbouring rows together: [i3][i1][i2]
+    v32[v32_xy ? ((int64_t)i3 * n1 + i1) * n2 + i2 : t] = (float)x;
     const float hi = __double2float_rn(x);
     vdf[t] = make_float2(hi, __double2float_rn(x - (double)hi));
   }
@@ -419,7 +424,7 @@ pwh_status pwh_set_potential(pwh_system* sys, const double* v_r, int32_t on_devi
       src = tmp;
     }
     k_potential_layout<<<1024, 256, 0, s.stream>>>(src, s.n1, s.n2, s.n3, 1.0 / (double)tot,
-                                                  s.d_v64, s.d_v32, s.d_vdf);
+                                                  spec_box(s) ? 1 : 0, s.d_v64, s.d_v32, s.d_vdf);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (tmp) {
