@@ -58,8 +58,8 @@ typedef enum {
                          36, 40, 48, 50, 60, 72, 80, 90, 96, 120, 144), which
                          compute in double-float (pairs of FP32 numbers, 48
                          significant bits, about 2^-46 relative rounding per
-                         operation), and the large GEMMs (exact integer-slice
-                         products on the tensor cores) */
+                         operation), and the large GEMMs (62-bit integers, exact
+                         products by residues on the tensor cores) */
   PWH_MIXED = 1,      /* FFT + potential in FP32; projector GEMMs on the BF16
                          tensor cores with FP32 accumulation, each operand split
                          into two BF16 terms (hi*hi + hi*lo + lo*hi, about 16
@@ -440,8 +440,8 @@ typedef struct {
   char name[32];     /* family: fft_z_inverse_fp64|fp32, fft_plane_fp64|fp32,
                         fft_z_forward_fp64|fp32, tc_gemm_becp, tc_gemm_backproj,
                         cgemm_fp64, cgemm_fp32, jacobi_fp64, cholqr_fp64,
-                        jacobi_fp32, zgemm_fp64_tc (sliced FP64-equivalent
-                        GEMM), zgemm_fp32_tc (three-slice FP32-equivalent
+                        jacobi_fp32, zgemm_fp64_tc (FP64-equivalent GEMM by
+                        residues), zgemm_fp32_tc (three-slice FP32-equivalent
                         GEMM) */
   int64_t launches;  /* timed launches (bracketed groups) */
   double total_ms;   /* summed device time */
@@ -488,8 +488,9 @@ pwh_status pwh_batch_davidson_solve(int32_t n, pwh_system* const* systems,
  * Jacobi: sweeps in FP32 to FP32 convergence (in one 16-CTA cluster with the
  * matrix in distributed shared memory when it fits there, n up to about 440),
  * then, for precision = PWH_FP64, the accumulated basis made unitary in FP64
- * (Newton-Schulz), Q^H H Q in FP64 and FP64 sweeps until
- * max|A_ij| <= 1e-13 max|A_ii|; for PWH_MIXED the FP32 result (one FP32
+ * (Newton-Schulz), Q^H H Q in FP64 and FP64 sweeps (n >= 256: one sweep, then
+ * quadratic refinement by matrix products) until max|A_ij| <= 1e-13 max|A_ii|;
+ * for PWH_MIXED the FP32 result (one FP32
  * Newton-Schulz step; eigenvalues to about 1e-7 ||H||), as the reduced-precision
  * phase of pwh_davidson_solve uses.  Asynchronous on the system's stream;
  * n <= 4096; another precision gives PWH_ERR_ARG. */
@@ -517,8 +518,8 @@ pwh_status pwh_subspace_cholqr(pwh_system* sys, int32_t precision, int32_t k, co
  * uses it: C = alpha op(A) B + beta C, op(A) = A^H when conj_a else A; op(A)
  * is M x K, B is K x N, C is M x N; all DEVICE complex128, column-major with
  * the given leading dimensions (lda >= rows of A as stored).  alpha, beta:
- * HOST double[2] (re, im).  precision PWH_FP64: FP64 arithmetic (products of
- * at least 2e8 flops as exact integer-slice products on the tensor cores);
+ * HOST double[2] (re, im).  precision PWH_FP64: FP64 arithmetic (large
+ * products as exact integer products by residues on the tensor cores);
  * PWH_MIXED: operands rounded to FP32, FP32 accumulation (relative error about
  * sqrt(K) 1e-7), result widened (products of at least 4e8 flops and 48
  * columns of A^H B or 96 of A B, or 1 and 16 columns when K (A^H B) or M (A B)

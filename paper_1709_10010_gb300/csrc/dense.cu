@@ -1531,11 +1531,11 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
 // within lim^2 of unitary (clusters of three and more equal eigenvalues are
 // resolved a pair at a time, or left to the Jacobi sweeps).
 //   Bound: four n x n products a step (12 in all) and one Jacobi sweep before
-// them, against two to three (30 in large clusters) sweeps of n - 1 grid-wide
-// rounds on the FP64 pipe (60 us a round at n = 1088).  The whole FP64
-// eigensolve, FP32 stage included: n = 1088 137 -> 87 ms, 1632 587 -> 249, 408
-// 21.7 -> 16.4, 256 10.4 -> 9.6, five 128-fold levels 311 -> 41; eigenvectors
-// orthonormal to 3e-15 instead of 1e-13.  Without the first sweep (three
+// them (k_jacobi_pair_sweep), against two to three (30 in large clusters) sweeps
+// of n - 1 grid-wide rounds on the FP64 pipe (60 us a round at n = 1088).  The
+// whole FP64 eigensolve, FP32 stage included: n = 1088 137 -> 42 ms, 1632 587 ->
+// 126, 408 21.7 -> 14.0, 256 10.4 -> 8.3, five 128-fold levels 311 -> 31;
+// eigenvectors orthonormal to 3e-15 instead of 1e-13.  Without the first sweep (three
 // refinement steps from the FP32 basis) n = 1088 takes 20 ms to the same
 // accuracy, but with eigenvector phases that differ by 1e-6 from the cyclic
 // sweeps'.  Below kRefineMinN the products run on the FP64 pipe and gain
@@ -1552,7 +1552,10 @@ struct RefineWs {
   unsigned long long* mx;  // max |F_ij|, max |F_ii| as ordered bit patterns
   int* done;               // 1: every off-diagonal element below the target
 };
-static size_t refine_bytes(int n) { return (size_t)n * 56 + 64; }
+static size_t refine_bytes(int n) {
+  // refinement arrays, then the pair sweep's two diagonals and rotations
+  return (size_t)n * 56 + 64 + (size_t)n * 16 + (size_t)(n / 2 + 1) * 20 + 64;
+}
 static RefineWs refine_carve(void* base, int n) {
   RefineWs w;
   w.s = (double2*)(((uintptr_t)base + 15) & ~(uintptr_t)15);
@@ -1762,6 +1765,232 @@ __global__ void __launch_bounds__(128) k_refine_m(double2* __restrict__ S,
   }
 }
 
+// ---- the first FP64 sweep in FP32 pairs ---------------------------------------
+// One cyclic sweep (the rounds and rotations of k_jacobi<double>) on the almost
+// diagonal A: its diagonal in FP64, off-diagonal elements and Q as pairs hi + lo of
+// FP32 numbers (48 bits).  A rotation is the identity plus a small correction, so a
+// new element is the old pair plus a correction formed in FP32 (angles of 1e-4 of
+// the element; the rotation angles themselves in FP64): what the refinement that
+// follows needs, a unitary basis to 1e-7 or better, at the FP32 pipes' rate.
+//   Each block computes its share of a round's rotations (k_jacobi computes them
+// all in every block: at n = 1088 some 25 of its 60 us a round on the FP64 pipe)
+// and publishes them; a second grid barrier separates them from the update.
+//   Bound: two grid barriers a round and the L2 traffic between them (A read by
+// halves and written, Q read and written: 66 MB a round at n = 1088).  The whole
+// eigensolve with this sweep in place of an FP64 one: n = 1088 86.8 -> 41.8 ms (42
+// of the 60 us a round), 1632 249 -> 126, 408 16.4 -> 14.0, 256 9.6 -> 8.3.
+struct PairRot {
+  float c1, sx, sy;    // c - 1, s
+  float sxl, syl;      // low parts of s
+};
+struct PairSweepArgs {
+  float4* A[2];   // (re hi, re lo, im hi, im lo), column-major
+  float4* Q;
+  double* d[2];   // diagonal
+  PairRot* rot;
+  int n, np;
+  GridBar gb;
+};
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
+  // two-sum of hi and x, then the low part: no contraction anywhere
+  const float s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb));
+  const float l = __fadd_rn(lo, e);
+  hi = __fadd_rn(s, l);
+  lo = __fsub_rn(l, __fsub_rn(hi, s));
+}
+__device__ __forceinline__ float4 pair_add(float4 a, float dx, float dy) {
+  pair_add(a.x, a.y, dx);
+  pair_add(a.z, a.w, dy);
+  return a;
+}
+__device__ __forceinline__ float4 pair_from(double2 v) {
+  const float xh = __double2float_rn(v.x), yh = __double2float_rn(v.y);
+  return make_float4(xh, __double2float_rn(v.x - (double)xh), yh, __double2float_rn(v.y - (double)yh));
+}
+// A and Q to pairs (in place: 16 bytes either way), the diagonal apart
+__global__ void k_pair_in(double2* A, double2* Q, int n, double* __restrict__ d) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= (int64_t)n * n) return;
+  const double2 a = A[t];
+  if (t % n == t / n) d[t / n] = a.x;
+  ((float4*)A)[t] = pair_from(a);
+  ((float4*)Q)[t] = pair_from(Q[t]);
+}
+__global__ void k_pair_out(const float4* Q, int64_t nn, double2* __restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nn) return;
+  const float4 q = Q[t];
+  out[t] = make_double2((double)q.x + (double)q.y, (double)q.z + (double)q.w);
+}
+
+constexpr int kPairThreads32 = 512;
+__global__ void __launch_bounds__(kPairThreads32, 1) k_jacobi_pair_sweep(PairSweepArgs a) {
+  extern __shared__ __align__(16) unsigned char jsm[];
+  const int n = a.n, np = a.np, P = np / 2;
+  PairRot* rot = (PairRot*)jsm;   // P
+  int* pp = (int*)(rot + P);      // P
+  int* pq = pp + P;               // P
+  unsigned epoch = 0;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+  const int Pe = P + (P & 1);     // folded triangle: Pe / 2 rows of Pe + 1
+  const int nA = (Pe / 2) * (Pe + 1), nQ = n * P;
+  for (int r = 0; r < np - 1; ++r) {
+    const int cur = r & 1;
+    const float4* A = a.A[cur];
+    const double* d = a.d[cur];
+    // a few rotations a block: they are long chains of FP64 operations
+    for (int k = blockIdx.x + gridDim.x * threadIdx.x; k < P; k += nth) {
+      int p = rr_player(k, r, np), q = rr_player(np - 1 - k, r, np);
+      if (p > q) { const int t = p; p = q; q = t; }
+      double c = 1.0;
+      double2 s = make_double2(0, 0);
+      if (p < n) {
+        const double app = d[p];
+        double dp = app;
+        if (q < n) {
+          const float4 v = A[(size_t)q * n + p];
+          const double2 apq = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+          const double aqq = d[q];
+          jacobi_rotation<double>(apq, app, aqq, c, s);
+          // J^H A J: the diagonal moves by t |A_pq| = Re(conj(s) A_pq) / c
+          const double sh = (s.x * apq.x + s.y * apq.y) / c;
+          dp = app - sh;
+          a.d[cur ^ 1][q] = aqq + sh;
+        }
+        a.d[cur ^ 1][p] = dp;
+      }
+      PairRot o;
+      const double s2 = s.x * s.x + s.y * s.y;
+      o.c1 = (float)(-s2 / (1.0 + c));  // c - 1 without cancellation
+      o.sx = (float)s.x;
+      o.sy = (float)s.y;
+      o.sxl = (float)(s.x - (double)o.sx);
+      o.syl = (float)(s.y - (double)o.sy);
+      a.rot[k] = o;
+    }
+    if (!grid_sync(a.gb, epoch)) return;
+    for (int k = threadIdx.x; k < P; k += blockDim.x) {
+      int p = rr_player(k, r, np), q = rr_player(np - 1 - k, r, np);
+      if (p > q) { const int t = p; p = q; q = t; }
+      pp[k] = p;
+      pq[k] = q;
+      // written by other blocks before the barrier: past the L1 cache
+      const float* g = &a.rot[k].c1;
+      rot[k] = PairRot{__ldcg(g), __ldcg(g + 1), __ldcg(g + 2), __ldcg(g + 3), __ldcg(g + 4)};
+    }
+    __syncthreads();
+    float4* An = a.A[cur ^ 1];
+    for (int t = tid; t < nA + nQ; t += nth) {
+      if (t < nA) {
+        // folded: row f holds column l = Pe - 1 - f (its k = 0 .. l), then l = f
+        const int f = t / (Pe + 1), u = t - f * (Pe + 1);
+        const int l = u < Pe - f ? Pe - 1 - f : f, k = u < Pe - f ? u : u - (Pe - f);
+        if (l >= P) continue;  // (k <= l)
+        const int pk = pp[k], qk = pq[k], pl = pp[l], ql = pq[l];
+        if (pk >= n || pl >= n) continue;
+        const bool vk = qk < n, vl = ql < n;
+        if (k == l) {
+          if (vk) An[(size_t)qk * n + pk] = An[(size_t)pk * n + qk] = make_float4(0.f, 0.f, 0.f, 0.f);
+          continue;
+        }
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a00 = A[(size_t)pl * n + pk];
+        const float4 a01 = vl ? A[(size_t)ql * n + pk] : z;
+        const float4 a10 = vk ? A[(size_t)pl * n + qk] : z;
+        const float4 a11 = (vk && vl) ? A[(size_t)ql * n + qk] : z;
+        const PairRot rk = rot[k], rl = rot[l];
+        // corrections d = A J - A by columns, then J^H (.) - (.) by rows
+        auto col = [&](float4 x, float4 y, float2& dx, float2& dy) {
+          dx.x = rl.c1 * x.x - (rl.sx * y.x + rl.sy * y.z);
+          dx.y = rl.c1 * x.z - (rl.sx * y.z - rl.sy * y.x);
+          dy.x = rl.c1 * y.x + (rl.sx * x.x - rl.sy * x.z);
+          dy.y = rl.c1 * y.z + (rl.sx * x.z + rl.sy * x.x);
+        };
+        float2 d00, d01, d10, d11;
+        col(a00, a01, d00, d01);
+        col(a10, a11, d10, d11);
+        auto row = [&](float4 x0, float2 e0, float4 x1, float2 e1, float2& o0, float2& o1) {
+          const float2 u0 = make_float2(x0.x + e0.x, x0.z + e0.y), u1 = make_float2(x1.x + e1.x, x1.z + e1.y);
+          o0.x = e0.x + (rk.c1 * u0.x - (rk.sx * u1.x - rk.sy * u1.y));
+          o0.y = e0.y + (rk.c1 * u0.y - (rk.sx * u1.y + rk.sy * u1.x));
+          o1.x = e1.x + (rk.c1 * u1.x + (rk.sx * u0.x + rk.sy * u0.y));
+          o1.y = e1.y + (rk.c1 * u1.y + (rk.sx * u0.y - rk.sy * u0.x));
+        };
+        float2 y00, y01, y10, y11;
+        row(a00, d00, a10, d10, y00, y10);
+        row(a01, d01, a11, d11, y01, y11);
+        auto put = [&](int i, int j, float4 v, float2 e) {
+          v = pair_add(v, e.x, e.y);
+          An[(size_t)j * n + i] = v;
+          An[(size_t)i * n + j] = make_float4(v.x, v.y, -v.z, -v.w);
+        };
+        put(pk, pl, a00, y00);
+        if (vl) put(pk, ql, a01, y01);
+        if (vk) put(qk, pl, a10, y10);
+        if (vk && vl) put(qk, ql, a11, y11);
+      } else {
+        const int e = t - nA;
+        const int l = e / n, i = e - l * n;
+        const int pl = pp[l], ql = pq[l];
+        if (pl >= n || ql >= n) continue;
+        const PairRot c = rot[l];
+        float4* Qp = a.Q + (size_t)pl * n + i;
+        float4* Qq = a.Q + (size_t)ql * n + i;
+        const float4 q0 = *Qp, q1 = *Qq;
+        // s with its low part: a systematic error of s would turn the column
+        const float x0 = c.c1 * q0.x - ((c.sx * q1.x + c.sy * q1.z) + (c.sxl * q1.x + c.syl * q1.z));
+        const float y0 = c.c1 * q0.z - ((c.sx * q1.z - c.sy * q1.x) + (c.sxl * q1.z - c.syl * q1.x));
+        const float x1 = c.c1 * q1.x + ((c.sx * q0.x - c.sy * q0.z) + (c.sxl * q0.x - c.syl * q0.z));
+        const float y1 = c.c1 * q1.z + ((c.sx * q0.z + c.sy * q0.x) + (c.sxl * q0.z + c.syl * q0.x));
+        *Qp = pair_add(q0, x0, y0);
+        *Qq = pair_add(q1, x1, y1);
+      }
+    }
+    if (!grid_sync(a.gb, epoch)) return;
+  }
+}
+
+// One sweep on A (n x n, FP64 in, destroyed) and Q (FP64 in, pairs out); A1 a second
+// buffer, ws the diagonals and rotations (16-byte aligned to 8).
+static void pair_sweep(System& s, DenseWs& w, double2* A, double2* A1, double2* Q, int n, char* ws,
+                       cudaStream_t st) {
+  unsigned* ctl = (unsigned*)w.ctl;
+  PWH_CUDA(cudaMemsetAsync(ctl, 0, 3 * sizeof(unsigned), st));  // barrier words
+  const int np = n + (n & 1), P = np / 2;
+  PairSweepArgs a;
+  a.A[0] = (float4*)A;
+  a.A[1] = (float4*)A1;
+  a.Q = (float4*)Q;
+  a.d[0] = (double*)(((uintptr_t)ws + 15) & ~(uintptr_t)15);
+  a.d[1] = a.d[0] + n;
+  a.rot = (PairRot*)(a.d[1] + n);
+  a.n = n;
+  a.np = np;
+  a.gb.count = ctl;
+  a.gb.unused = ctl + 1;
+  a.gb.abort = (int*)(ctl + 2);
+  a.gb.err = device_error_word(s);
+  k_pair_in<<<(unsigned)(((int64_t)n * n + 255) / 256), 256, 0, st>>>(A, Q, n, a.d[0]);
+  PWH_LAUNCH_CHECK();
+  const size_t smem = (size_t)P * (sizeof(PairRot) + 2 * sizeof(int));
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_jacobi_pair_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (kJacobiMaxN / 2 + 1) * (int)(sizeof(PairRot) + 2 * sizeof(int)));
+  });
+  int dev = 0, nsm = 0, per_sm = 0;
+  PWH_CUDA(cudaGetDevice(&dev));
+  PWH_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  PWH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi_pair_sweep, kPairThreads32, smem));
+  const int64_t items = (int64_t)P * P / 2 + (int64_t)n * P;
+  const int want = (int)std::max<int64_t>(1, std::min<int64_t>((items + 511) / 512, nsm));
+  const int blocks = std::max(1, std::min(want, nsm * std::max(per_sm, 1)));
+  void* args[] = {&a};
+  PWH_CUDA(cudaLaunchCooperativeKernel((void*)k_jacobi_pair_sweep, blocks, kPairThreads32, args, smem, st));
+  note_launch();
+}
+
 static size_t jacobi_ws_bytes(size_t nn, int n) {
   // FP64: A0, A1, Q0, Q1, G;  FP32: a0, a1, q0, q1;  diagonal d;  the
   // refinement's per-index arrays
@@ -1913,8 +2142,9 @@ void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, in
     // steps, the target test with a last step, and Jacobi sweeps again only
     // where the target was missed.  The limits leave X unitary to 1e-15 in
     // clusters too, where angles up to them keep being applied.
-    launch_jacobi<double>(s, w, A0, A1, Q0, Q1, n, tol64, 1, out_buf, st);
-    // a sweep is an odd number of rounds: its result is in the second buffers
+    pair_sweep(s, w, A0, A1, Q0, n, (char*)(dg + n) + (((size_t)n * 56 + 64 + 15) & ~(size_t)15), st);
+    k_pair_out<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>((const float4*)Q0, (int64_t)nn, Q1);
+    PWH_LAUNCH_CHECK();
     const RefineWs rw = refine_carve(dg + n, n);
     double2 *X = Q1, *Gx = A0, *S = A1, *Gr = Q0, *Xn = G;
     const unsigned g1 = (unsigned)((n + 255) / 256);
