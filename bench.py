@@ -612,12 +612,13 @@ def run_batched(pwh, syn, torch, ncells=32, nthreads=16):
 
 
 # The FP64-accurate FFT passes of the compiled box sizes run in double-float
-# arithmetic (pairs of FP32 numbers) on the FP32 pipes: a double-float add is
-# 20 FP32 instructions, a multiply 7, and the nominal 5 N log2 N flops of a
-# transform are 6 adds and 4 multiplies in 10, so one FP64-equivalent flop
-# costs 14.8 FP32 instructions; the pipes issue 152 x 128 x 2.07e9 of those a
-# second (half the FP32 flop rate, which counts an FMA as two).
-DF_FP32_OPS_PER_FLOP = (6 * 20 + 4 * 7) / 10
+# arithmetic (pairs of FP32 numbers) on the FP32 pipes: a double-float sum is
+# 11 FP32 instructions, a complex product 40, and the nominal 5 N log2 N flops
+# of a radix-2 butterfly are one complex product and two complex sums in 10, so
+# one FP64-equivalent flop costs 8.4 FP32 instructions (transforms with fewer
+# products than nominal can pass this rate); the pipes issue 152 x 128 x 2.07e9
+# of those a second (half the FP32 flop rate, which counts an FMA as two).
+DF_FP32_OPS_PER_FLOP = (40 + 4 * 11) / 10
 DF_ALU_TFLOPS = FP32_ALU_TFLOPS / 2 / DF_FP32_OPS_PER_FLOP
 
 FAMILY_BOUND = {
@@ -627,7 +628,7 @@ FAMILY_BOUND = {
     "fft_z_inverse_fp64": ("alu", "flops", "df"), "fft_z_forward_fp64": ("alu", "flops", "df"),
     "tc_gemm_becp": ("tensor", "flops", "bf16"), "tc_gemm_backproj": ("tensor", "flops", "bf16"),
     "cgemm_fp64": ("alu", "flops", "fp64"), "cgemm_fp32": ("alu", "flops", "fp32"),
-    "jacobi_fp64": ("alu", "flops", "fp64"), "cholqr_fp64": ("alu", "flops", "fp64"),
+    "jacobi_fp64": ("alu", "flops", None), "cholqr_fp64": ("alu", "flops", "fp64"),
     "jacobi_fp32": ("alu", "flops", "fp32"), "zgemm_fp64_tc": ("tensor", "flops", "bf16"),
     "zgemm_fp32_tc": ("tensor", "flops", "bf16"),
 }
@@ -648,11 +649,9 @@ TRAFFIC_PER_LAUNCH = {    # family -> bytes per launch
     # predates the kernel's current phase-1 schedule and double buffering)
 }
 TRAFFIC_PER_FLOP = {      # family -> bytes per counted flop
-    # one 1088 x 544 x 16,384 FP64-equivalent product on the persistent
-    # tensor-core kernel (bench.py --gemm 1088,544,16384,fp64,1): 6.12 GB of
-    # DRAM traffic over its six kernels for 2.79e12 counted tensor flops
-    # (profiles/oz_gemm_fp64_conj_1088x544x16384.md)
-    "zgemm_fp64_tc": 6.118e9 / 2.7928e12,
+    # (the FP64-equivalent GEMM's capture, profiles/
+    # oz_gemm_fp64_conj_1088x544x16384.md, is of the slice-pair form that the
+    # residue form replaced)
 }
 
 
@@ -674,7 +673,11 @@ def family_roofline(fam, d, s=None):
         achieved = work / sec / 1e12
     elif key == "df":
         peak, unit = DF_ALU_TFLOPS, "TFLOP/s"
-        psrc = "derived double-float rate (FP32 instruction rate / 14.8)"
+        psrc = "derived double-float rate (FP32 instruction rate / 8.4)"
+        achieved = work / sec / 1e12
+    elif key is None:
+        peak, unit = None, "TFLOP/s"
+        psrc = "none (a sweep on the FP32 pipes, products on the tensor cores)"
         achieved = work / sec / 1e12
     else:
         peak, unit, psrc = FP64_ALU_TFLOPS, "TFLOP/s", "nominal FP64 rate"
