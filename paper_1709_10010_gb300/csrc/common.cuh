@@ -269,7 +269,7 @@ struct System {
   DevBuf<char> ws_grid;             // SCF steps: a real and a complex full-box grid
   DevBuf<char> ws_tune;             // scratch of the tile autotuner
   DevBuf<char> ws_tc;               // packed BF16 operands of the tensor-core path
-  DevBuf<char> ws_oz;               // sliced operands and partials of the FP64-equivalent GEMM
+  DevBuf<char> ws_oz;               // residues (FP64-equivalent GEMM), slices and partials (FP32-)
   int tc_nb_cap = 0, tc_P = -1;     // geometry the ws_tc zero padding was laid out for
   int* d_err = nullptr;             // device error word (bounded waits that gave up)
   float* d_mlp = nullptr;           // learned-preconditioner parameters

@@ -1777,8 +1777,11 @@ __global__ void __launch_bounds__(128) k_refine_m(double2* __restrict__ S,
 // and publishes them; a second grid barrier separates them from the update.
 //   Bound: two grid barriers a round and the L2 traffic between them (A read by
 // halves and written, Q read and written: 66 MB a round at n = 1088).  The whole
-// eigensolve with this sweep in place of an FP64 one: n = 1088 86.8 -> 41.8 ms (42
-// of the 60 us a round), 1632 249 -> 126, 408 16.4 -> 14.0, 256 9.6 -> 8.3.
+// eigensolve with this sweep in place of an FP64 one: n = 1088 86.8 -> 41.8 ms (60
+// -> 20 us a round), 1632 249 -> 126, 408 16.4 -> 14.0, 256 9.6 -> 8.3.  One barrier
+// a round (the next round's rotations formed by the threads that make their
+// elements) gave 18 us there but was slower at 256 to 320; four rows of Q in flight
+// a thread changed nothing.
 struct PairRot {
   float c1, sx, sy;    // c - 1, s
   float sxl, syl;      // low parts of s
