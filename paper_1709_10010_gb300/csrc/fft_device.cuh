@@ -15,19 +15,19 @@ namespace pwh {
 #define PWH_S5B 0.587785252292473129168705954639
 
 // z * (sg * i)
-template <typename T> __device__ __forceinline__ cx<T> rot(cx<T> z, T sg) {
+template <typename T> __host__ __device__ __forceinline__ cx<T> rot(cx<T> z, T sg) {
   return mk<T>(-sg * z.y, sg * z.x);
 }
 
 // In-register DFT of length R with sign sg (+1 inverse, -1 forward).
-template <typename T, int R> __device__ __forceinline__ void dft(cx<T>* a, T sg);
+template <typename T, int R> __host__ __device__ __forceinline__ void dft(cx<T>* a, T sg);
 
-template <typename T> __device__ __forceinline__ void dft2(cx<T>* a) {
+template <typename T> __host__ __device__ __forceinline__ void dft2(cx<T>* a) {
   cx<T> t = a[0];
   a[0] = add<T>(t, a[1]);
   a[1] = sub<T>(t, a[1]);
 }
-template <typename T, int R> __device__ __forceinline__ void dft(cx<T>* a, T sg) {
+template <typename T, int R> __host__ __device__ __forceinline__ void dft(cx<T>* a, T sg) {
   if constexpr (R == 2) {
     dft2<T>(a);
   } else if constexpr (R == 3) {

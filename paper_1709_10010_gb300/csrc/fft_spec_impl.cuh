@@ -135,21 +135,28 @@ template <typename T, int N> struct Fac {
   static_assert(N1 > 1 && N1 <= 16 && N2 <= 16, "factor");
   static constexpr int A = pfa ? N2 * inv_mod(N2, N1) % N : 1;
   static constexpr int B = pfa ? N1 * inv_mod(N1, N2) % N : N1;
-  __device__ static __forceinline__ int wrap(int i) { return i >= N ? i - N : i; }
-  __device__ static __forceinline__ int idx_a(int n1, int n2) {
+  __host__ __device__ static __forceinline__ int wrap(int i) { return i >= N ? i - N : i; }
+  __host__ __device__ static __forceinline__ int idx_a(int n1, int n2) {
     if constexpr (pfa) return wrap(N1 * n2 + N2 * n1);
     else return N2 * n1 + n2;
   }
-  __device__ static __forceinline__ int idx_b(int k1, int k2) {
+  __host__ __device__ static __forceinline__ int idx_b(int k1, int k2) {
     if constexpr (pfa) return wrap((A * k1) % N + (B * k2) % N);
     else return k1 + N1 * k2;
   }
 };
 
+// The arithmetic of edge N's double-float passes: the fused operations of fft_df.cuh
+// where the edge has coprime factors; 50 and 96 keep twiddles between their passes
+// and err 6% and 2% more with the fused operations than with the composed ones, so
+// they take those (dfa).
+struct dfa;
+template <int N> using DfPass = std::conditional_t<Fac<df, N>::pfa, df, dfa>;
+
 // The twiddle of the transform's sign: conjugated for forward ones (in
 // double-float a sign change; the other types keep the product by +-1, which
 // the compiler folds).
-template <typename T, bool INV> __device__ __forceinline__ cx<T> signed_tw(cx<T> w) {
+template <typename T, bool INV> __host__ __device__ __forceinline__ cx<T> signed_tw(cx<T> w) {
   if constexpr (is_df<T>) {
     if (!INV) w.y = -w.y;
   } else {
@@ -159,7 +166,7 @@ template <typename T, bool INV> __device__ __forceinline__ cx<T> signed_tw(cx<T>
 }
 
 template <typename T, int R, bool INV, int NT, int S>
-__device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
+__host__ __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
   constexpr CPlan P = make_cplan(R);
   if constexpr (S < P.ns) {
     constexpr int Rs = P.R[S], M = P.M[S], L = P.L[S];
@@ -189,7 +196,7 @@ __device__ __forceinline__ void reg_stages(cx<T>* a, const cx<T>* tw) {
 // In-register DFT of length R (natural order in and out) with sign +1 (INV)
 // or -1; tw[t] = exp(2 pi i t / NT), R | NT.
 template <typename T, int R, bool INV, int NT>
-__device__ __forceinline__ void dft_reg(cx<T>* x, const cx<T>* tw) {
+__host__ __device__ __forceinline__ void dft_reg(cx<T>* x, const cx<T>* tw) {
   constexpr int RA = R == 12 ? 4 : R == 6 || R == 10 ? 2 : R == 15 ? 3 : 1, RB = R / RA;
   if constexpr (few_products<T> && RA > 1) {
     // coprime factors: no twiddles (the maps of Fac)
@@ -569,13 +576,16 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
 }
 
 // Threads of a plane block.  Double-float threads hold 128 registers: two blocks
-// of 256 an SM, whose barriers then overlap with the other's arithmetic (90^3,
-// 128 bands: 2.92 ms, against 3.45 ms in one block of 512 and 3.90 in one of
-// 384).  FP32 waits for shared memory: 256 threads, two blocks an SM by shared
+// of 256 an SM, whose barriers then overlap with the other's arithmetic, up to 90,
+// one of 512 from 96 on, where the columns fill the SM's shared memory (64 bands,
+// blocks of 256 and 512: 40 152 and 187 us, 72 1.12 and 1.42 ms, 90 2.13 and 2.28,
+// 96 3.67 and 3.28, 120 6.43 and 5.79, 144 15.4 and 14.1).  FP32 waits for shared
+// memory: 256 threads, two blocks an SM by shared
 // memory, at 90^3 (0.461 ms for 128 bands, 0.470 with 512); one block of 1,024 where
 // the columns leave room for one (144^3, 512 bands: 8.28 ms, 8.43 with 512, 9.8 with
 // 768).
-template <typename T, int N> constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 120 ? 1024 : 256) : 256;
+template <typename T, int N>
+constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 120 ? 1024 : 256) : (N >= 96 ? 512 : 256);
 
 // Shared memory of the plane pass for `rows` rows per chunk.
 template <typename T, int N> constexpr size_t ks_plane_smem(int ncols, int rows) {

@@ -9,7 +9,7 @@ template <> bool spec_pass<df>(SpecPass pass, System& s, const PassArgs& a) {
   switch (s.n1) {
 #define PWH_SPEC_CASE(n)                                                               \
   case n:                                                                              \
-    spec_launch<std::conditional_t<n == 50, dfa, df>, n>(pass, s, a);                  \
+    spec_launch<DfPass<n>, n>(pass, s, a);                                             \
     return true;
     PWH_SPEC_SIZES(PWH_SPEC_CASE)
 #undef PWH_SPEC_CASE
