@@ -35,23 +35,25 @@ namespace pwh {
 // ------------------------------------------------------------- the moduli ----
 constexpr int kMod = 16;
 constexpr int kT = 62;  // operands are integers of 2-norm at most 2^kT
+constexpr int kDigits = 6;
 struct ModTab {
   int p[kMod];
   // 2^16, 2^32 and 2^48 mod p, symmetric: the weights of X's 16-bit limbs
   float c1[kMod], c2[kMod], c3[kMod], inv[kMod];
-  // (P/p)^-1 mod p over p as a 90-bit fraction, V / P = sum r_i K_i mod 1: its
+  // (P/p)^-1 mod p over p as a 108-bit fraction, V / P = sum r_i K_i mod 1: its
   // 18-bit digits, leading first
-  int k[kMod][5];
-  double scale;  // P 2^(-2 kT - 1)
+  int k[kMod][kDigits];
+  unsigned long long ph;  // P 2^-kPShift, rounded: in [2^63, 2^64)
 };
+constexpr int kPShift = 62;
 constexpr ModTab make_mod_tab() {
   ModTab t{};
   const int p[kMod] = {256, 255, 253, 251, 247, 241, 239, 233,
                        229, 227, 223, 217, 211, 199, 197, 193};
-  double P = 1.0;
+  unsigned __int128 P = 1;  // 2^125.37
   for (int i = 0; i < kMod; ++i) {
     t.p[i] = p[i];
-    P *= p[i];
+    P *= (unsigned)p[i];
     long long w = 1 << 16;
     auto sym = [&](long long v) {
       v %= p[i];
@@ -66,20 +68,19 @@ constexpr ModTab make_mod_tab() {
       if (j != i) rest = rest * p[j] % p[i];
     long long iv = 1;
     while (rest * iv % p[i] != 1) ++iv;
-    // iv 2^90 / p by long division
+    // iv 2^108 / p by long division
     long long rem = iv;
-    for (int k = 0; k < 5; ++k) {
+    for (int k = 0; k < kDigits; ++k) {
       rem <<= 18;
       t.k[i][k] = (int)(rem / p[i]);
       rem %= p[i];
     }
   }
-  double s = P;
-  for (int k = 0; k < 2 * kT + 1; ++k) s *= 0.5;
-  t.scale = s;
+  t.ph = (unsigned long long)((P + ((unsigned __int128)1 << (kPShift - 1))) >> kPShift);
   return t;
 }
 constexpr ModTab kTab = make_mod_tab();
+static_assert(kTab.ph >> 63, "P 2^-kPShift has 64 bits");
 __constant__ float c_mod_p[kMod] = {256, 255, 253, 251, 247, 241, 239, 233,
                                     229, 227, 223, 217, 211, 199, 197, 193};
 constexpr float kMagic = 12582912.f;  // 1.5 2^23: adding it rounds to an integer
@@ -214,6 +215,16 @@ template <int I> __device__ __forceinline__ float mod_res(const float* l) {
   constexpr float p = (float)kTab.p[I], inv = kTab.inv[I];
   constexpr float c1 = kTab.c1[I], c2 = kTab.c2[I], c3 = kTab.c3[I];
   return mod_sym(fmaf(l[3], c3, fmaf(l[2], c2, fmaf(l[1], c1, l[0]))), p, inv);
+}
+// four residues, first reduced to |.| <= p / 2, as signed bytes (128 and -128 of
+// p = 256 are the same byte)
+__device__ __forceinline__ unsigned pack_res(const float* x, float p) {
+  const float top = 0.5f * (p - 1.f);
+  unsigned b[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    b[u] = __float_as_uint((x[u] > top ? x[u] - p : x[u] < -top ? x[u] + p : x[u]) + kMagic);
+  return __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
 }
 // two small integers as BF16 (their FP32 patterns have 16 zero trailing bits)
 __device__ __forceinline__ unsigned pack_bf16(float a, float b) {
@@ -585,39 +596,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 }
 
 // ---------------------------------------------------------- reconstruction ----
-// V / P as a fraction (mod 1).  The symmetric residues of one K range times
-// the 18-bit digits of the constants, in 32-bit multiply-adds (16 residues of at
-// most 256, the sum of two: below 2^31; 64-bit multiply-adds on 31-bit digits
-// ran at a quarter of their rate), then carried into a 96-bit fraction, to which
-// every K range adds.  Opposite residues cancel exactly.
+// V / P as a fraction (mod 1): the symmetric residues times the 18-bit digits of the
+// constants, in 32-bit multiply-adds (16 residues of at most 256, the sum of two:
+// below 2^31; 64-bit multiply-adds on 31-bit digits ran at a quarter of their rate),
+// then carried into a 96-bit fraction.  Residues of several K ranges are added modulo
+// p first, and those of two products added as they are: a product that is zero has
+// residues that are all zero.  The fraction is off by at most 2^-95, 2^-94 of |a| |b|:
+// products of integers come out exact up to where |a| |b| passes 2^40 times the
+// result (2^24 with five digits).
 struct CrtDigits {
-  int d[5] = {0, 0, 0, 0, 0};
+  int d[kDigits] = {0, 0, 0, 0, 0, 0};
   template <int I> __device__ __forceinline__ void add(int r) {
     constexpr int k0 = kTab.k[I][0], k1 = kTab.k[I][1], k2 = kTab.k[I][2], k3 = kTab.k[I][3],
-                  k4 = kTab.k[I][4];
+                  k4 = kTab.k[I][4], k5 = kTab.k[I][5];
     d[0] += r * k0;
     d[1] += r * k1;
     d[2] += r * k2;
     d[3] += r * k3;
     d[4] += r * k4;
+    d[5] += r * k5;
   }
 };
-struct CrtAcc {
-  unsigned long long h = 0;  // leading 64 bits
-  unsigned l = 0;            // 32 more
-  __device__ __forceinline__ void add(const CrtDigits& c) {
+struct CrtFrac {
+  unsigned long long h;  // leading 64 bits
+  unsigned l;            // 32 more
+  __device__ __forceinline__ void set(const CrtDigits& c) {
     constexpr int M = (1 << 18) - 1;
-    const int t3 = c.d[3] + (c.d[4] >> 18), t2 = c.d[2] + (t3 >> 18), t1 = c.d[1] + (t2 >> 18),
-              t0 = c.d[0] + (t1 >> 18);
-    const unsigned d1 = t1 & M, d2 = t2 & M, d3 = t3 & M, d4 = c.d[4] & M;
+    const int t4 = c.d[4] + (c.d[5] >> 18), t3 = c.d[3] + (t4 >> 18), t2 = c.d[2] + (t3 >> 18),
+              t1 = c.d[1] + (t2 >> 18), t0 = c.d[0] + (t1 >> 18);
+    const unsigned d1 = t1 & M, d2 = t2 & M, d3 = t3 & M, d4 = t4 & M, d5 = c.d[5] & M;
     const unsigned hi = ((unsigned)t0 << 14) | (d1 >> 4);
     const unsigned lo = (d1 << 28) | (d2 << 10) | (d3 >> 8);
-    const unsigned ll = (d3 << 24) | (d4 << 6);
-    const unsigned s = l + ll;
-    h += (((unsigned long long)hi << 32) | lo) + (s < ll ? 1u : 0u);
-    l = s;
+    h = ((unsigned long long)hi << 32) | lo;
+    l = (d3 << 24) | (d4 << 6) | (d5 >> 12);
   }
-  // the signed value times 2^(ea + eb - 2 kT)
+  // the signed value times 2^(ea + eb - 2 kT), rounded once: the truncations
+  // below add up to less than 2^-61 of it
   __device__ __forceinline__ double value(int ea, int eb) const {
     const bool neg = (long long)h < 0;
     const unsigned lx = neg ? 0u - l : l;
@@ -632,14 +646,18 @@ struct CrtAcc {
       s = __clzll((long long)hx);
       w = s ? (hx << s) | (((unsigned long long)lx << 32) >> (64 - s)) : hx;
     }
-    // w in [2^63, 2^64), rounded to a double in [1, 2] by integer operations
-    // (conversions issue on the narrow FP64 pipe); V 2^(-2 kT) = w 2^(-64 - s)
-    // P 2^(-2 kT)
-    const unsigned long long r = (w >> 11) + ((w >> 10) & 1);  // 2^52 .. 2^53
-    const double u = __longlong_as_double((long long)(r + (1022ull << 52)));
-    constexpr double scale = kTab.scale;
-    double d = u * scale;
-    const int sc = ea + eb - s, ed = (int)((__double2hiint(d) >> 20) & 0x7ff);
+    // |V| = w 2^(-64 - s) P = (w ph 2^-64) 2^(kPShift - s), by integer operations
+    // (conversions and products in FP64 issue on the narrow FP64 pipe)
+    unsigned long long q = __umul64hi(w, kTab.ph);  // 2^62 .. 2^64
+    if (!(q >> 63)) {
+      q += q;
+      ++s;
+    }
+    // to 53 bits; a double in [1, 2]
+    const unsigned long long r = (q >> 11) + ((q >> 10) & 1);  // 2^52 .. 2^53
+    double d = __longlong_as_double((long long)(r + (1022ull << 52)));
+    const int sc = ea + eb - s + (kPShift + 63 - 2 * kT);
+    const int ed = (int)((__double2hiint(d) >> 20) & 0x7ff);
     if (ed + sc >= 1 && ed + sc <= 2046)
       d = __hiloint2double(__double2hiint(d) + (sc << 20), __double2loint(d));
     else
@@ -673,10 +691,10 @@ __device__ __forceinline__ void crt_store(const CrtOut& o, double re, double im,
 // rows 2m, 2m+1 and columns 2n, 2n+1 (Re = C[2m][2n] + C[2m+1][2n+1], Im =
 // C[2m][2n+1] - C[2m+1][2n]); op(A) = A: (C[m][2n], C[m][2n+1]).  A block takes
 // 32 m (a warp's lanes: coalesced C) by NB n, its residues through shared
-// memory (16-byte loads, all in flight; pitch of an odd number of words): per
-// thread two neighbouring n at a time (20,000 x 544 outputs: 0.24 ms; 530
+// memory (16-byte loads, all in flight; pitch of an odd number of words), those of
+// several K ranges (RANGES) added modulo p on the way (20,000 x 544 outputs: 0.24 ms; 530
 // instructions an output, FP64 pipe 48% and issue slots 60% busy).
-template <bool CONJ>
+template <bool CONJ, bool RANGES>
 __global__ void __launch_bounds__(256, 3)
     k_mod_crt(const unsigned char* __restrict__ res, int nz, int M, int N, int64_t Np,
               const int* __restrict__ exa, const int* __restrict__ exb,
@@ -688,61 +706,72 @@ __global__ void __launch_bounds__(256, 3)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int m = blockIdx.x * 32 + lane, n0 = blockIdx.y * NB;
   const int64_t rows = (CONJ ? 2 : 1) * (int64_t)M;
-  CrtAcc re[2 * PAIRS], im[2 * PAIRS];
-  for (int z = 0; z < nz; ++z) {
-    if (z) __syncthreads();
-    {
-      // 128 chunks of 16 bytes a modulus, eight moduli a thread
-      const int c = threadIdx.x & 127, r = c / (RW / 4), q = c % (RW / 4);
-      const int64_t row = (int64_t)blockIdx.x * ROWS + r, col = 2 * (int64_t)n0 + 16 * q;
+  {
+    // 128 chunks of 16 bytes a modulus, eight moduli a thread
+    const int c = threadIdx.x & 127, r = c / (RW / 4), q = c % (RW / 4), odd = threadIdx.x >> 7;
+    const int64_t row = (int64_t)blockIdx.x * ROWS + r, col = 2 * (int64_t)n0 + 16 * q;
+    const bool in = row < rows && col < Np;
+    auto at = [&](int z, int mod) {
+      return in ? __ldg((const uint4*)(res + (((size_t)z * kMod + mod) * rows + row) * Np + col))
+                : make_uint4(0, 0, 0, 0);
+    };
+    auto put = [&](int mod, uint4 v) {
+      unsigned* d = sm + (mod * ROWS + r) * PW + 4 * q;
+      d[0] = v.x;
+      d[1] = v.y;
+      d[2] = v.z;
+      d[3] = v.w;
+    };
+    if constexpr (!RANGES) {
       uint4 v[8];
-      const bool in = row < rows && col < Np;
 #pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = at(0, 2 * i + odd);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) put(2 * i + odd, v[i]);
+    } else {
+#pragma unroll 1
       for (int i = 0; i < 8; ++i) {
-        const int mod = 2 * i + (threadIdx.x >> 7);
-        v[i] = in ? __ldg((const uint4*)(res + (((size_t)z * kMod + mod) * rows + row) * Np + col))
-                  : make_uint4(0, 0, 0, 0);
-      }
+        const int mod = 2 * i + odd;
+        const float p = c_mod_p[mod], inv = 1.f / p;
+        int t[16] = {};
+#pragma unroll 4
+        for (int z = 0; z < nz; ++z) {
+          const uint4 v = at(z, mod);
+          const unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        unsigned* d = sm + ((2 * i + (threadIdx.x >> 7)) * ROWS + r) * PW + 4 * q;
-        d[0] = v[i].x;
-        d[1] = v[i].y;
-        d[2] = v[i].z;
-        d[3] = v[i].w;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int pr = 0; pr < PAIRS; ++pr) {
-      CrtDigits dr[2], di[2];
-      const unsigned* p = sm + (CONJ ? 2 : 1) * lane * PW + warp * PAIRS + pr;
-      each_mod<0>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        const unsigned x = p[i * ROWS * PW];
-        unsigned y = 0;
-        if constexpr (CONJ) y = p[i * ROWS * PW + PW];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int a0 = (signed char)(x >> (16 * u)), a1 = (signed char)(x >> (16 * u + 8));
-          if constexpr (CONJ) {
-            const int b0 = (signed char)(y >> (16 * u)), b1 = (signed char)(y >> (16 * u + 8));
-            dr[u].template add<i>(a0 + b1);
-            di[u].template add<i>(a1 - b0);
-          } else {
-            dr[u].template add<i>(a0);
-            di[u].template add<i>(a1);
-          }
+          for (int u = 0; u < 16; ++u) t[u] += (signed char)(w[u / 4] >> (8 * (u % 4)));
         }
-      });
+        float x[16];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        re[2 * pr + u].add(dr[u]);
-        im[2 * pr + u].add(di[u]);
+        for (int u = 0; u < 16; ++u) x[u] = mod_sym((float)t[u], p, inv);
+        put(mod, make_uint4(pack_res(x, p), pack_res(x + 4, p), pack_res(x + 8, p), pack_res(x + 12, p)));
       }
     }
   }
+  __syncthreads();
   if (m >= M) return;
+  const unsigned* mine = sm + (CONJ ? 2 : 1) * lane * PW + warp * PAIRS;
+  CrtFrac re[2 * PAIRS], im[2 * PAIRS];
+#pragma unroll
+  for (int u = 0; u < 2 * PAIRS; ++u) {
+    CrtDigits dr, di;
+    const unsigned* p = mine + u / 2;
+    each_mod<0>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      const unsigned x = p[i * ROWS * PW] >> (16 * (u & 1));
+      const int a0 = (signed char)x, a1 = (signed char)(x >> 8);
+      if constexpr (CONJ) {
+        const unsigned y = p[i * ROWS * PW + PW] >> (16 * (u & 1));
+        dr.template add<i>(a0 + (signed char)(y >> 8));
+        di.template add<i>(a1 - (signed char)y);
+      } else {
+        dr.template add<i>(a0);
+        di.template add<i>(a1);
+      }
+    });
+    re[u].set(dr);
+    im[u].set(di);
+  }
   const int ea = exa[m];
   const double rs = rowscale ? rowscale[m] : 1.0;
 #pragma unroll
@@ -959,12 +988,14 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
   o.mode = pm1 && alpha.x == 1.0 && beta.x == 0.0 && beta.y == 0.0 ? 0
            : pm1 && beta.x == 1.0 && beta.y == 0.0                 ? 1
                                                                    : 2;
+  const dim3 gc((M + 31) / 32, conjA ? (N + 15) / 16 : (N + 31) / 32);
+  auto crt = [&](auto kernel) {
+    kernel<<<gc, 256, 0, st>>>(res, g.nz, M, N, g.Np, exa, exb, rowscale, o, C, ldc);
+  };
   if (conjA)
-    k_mod_crt<true><<<dim3((M + 31) / 32, (N + 15) / 16), 256, 0, st>>>(res, g.nz, M, N, g.Np, exa, exb,
-                                                                      rowscale, o, C, ldc);
+    g.nz > 1 ? crt(k_mod_crt<true, true>) : crt(k_mod_crt<true, false>);
   else
-    k_mod_crt<false><<<dim3((M + 31) / 32, (N + 31) / 32), 256, 0, st>>>(res, g.nz, M, N, g.Np, exa, exb,
-                                                                       rowscale, o, C, ldc);
+    g.nz > 1 ? crt(k_mod_crt<false, true>) : crt(k_mod_crt<false, false>);
   PWH_LAUNCH_CHECK();
 }
 
