@@ -28,12 +28,12 @@
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "gemm_mod_geom.cuh"
 #include "tc_ptx.cuh"
 
 namespace pwh {
 
 // ------------------------------------------------------------- the moduli ----
-constexpr int kMod = 16;
 constexpr int kT = 62;  // operands are integers of 2-norm at most 2^kT
 constexpr int kDigits = 6;
 struct ModTab {
@@ -351,7 +351,7 @@ struct ModArgs {
   int bn;            // tile width: a multiple of 32, at most 256
   int gm, gn, gz;    // tiles and K ranges
   int kb_total, kb_per;  // 64-wide K blocks, and a K range's share
-  int z0;            // first K range's index in the output
+  int accum;         // add to the residues of the earlier K segments
   int64_t Np;        // output pitch (bytes): gn bn
   unsigned char* out;  // [z][modulus][m][n]
   int* err;
@@ -523,9 +523,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       const int n0 = (rem % args.gn) * args.bn + half * 128;
       const int kb0 = z * args.kb_per, kb_end = min(args.kb_total, kb0 + args.kb_per);
       const float p = c_mod_p[mod], inv = 1.f / p;
+      // this thread's residues, one byte each, a row's columns side by side: 16-byte
+      // accesses (a byte store a column, with the rows of a warp side by side, took
+      // 45k clocks a tile, more than a short K's MMAs)
+      unsigned char* o = args.out + (((size_t)z * kMod + mod) * args.Mr + m) * args.Np + n0;
       float acc[128];
 #pragma unroll
       for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+      if (args.accum && m < args.Mr) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          if (c * 16 < hn) {
+            const uint4 w = *(const uint4*)(o + c * 16);
+            const unsigned v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int u = 0; u < 16; ++u) acc[c * 16 + u] = (float)(signed char)(v[u / 4] >> (8 * (u % 4)));
+          }
+        }
+      }
       for (int kc = kb0; kc < kb_end; kc += kChunkKb, ++lc) {
         const int buf = lc & 1;
         if (!mbar_wait(&tfull[buf], (lc >> 1) & 1, abort_flag)) {
@@ -550,11 +565,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       }
       if (!ok) break;
       if (m < args.Mr) {
-        // symmetric residues, one byte each, a row's columns side by side:
-        // 16-byte stores (a byte store a column, with the rows of a warp side
-        // by side, took 45k clocks a tile, more than a short K's MMAs)
-        unsigned char* o = args.out +
-                           (((size_t)(args.z0 + z) * kMod + mod) * args.Mr + m) * args.Np + n0;
         const float top = 0.5f * (p - 1.f);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -819,107 +829,16 @@ static int mod_pairs() {
   return pairs;
 }
 
-// Geometry of one product: K segments whose residues fit the workspace (their
-// residues add up modulo p: one rounding whatever the segments), K ranges of a
-// segment that spread few tiles over the GPU.
-constexpr size_t kOzSliceCap = (size_t)3 << 30;
-struct ModGeom {
-  int64_t Mr, Nr, Np;
-  int bn, gm, gn;
-  int kseg;       // complex K per segment
-  int nseg;
-  int64_t seg;    // real K of a segment, padded to 64
-  int kb, kb_per, gz, nz;  // K blocks, blocks a range, ranges a segment / in all
-  int Sa, Sb;     // blocks per row norm
-  size_t bytes_a, bytes_b, bytes_r, bytes_n, bytes_e;
-  size_t total() const { return bytes_a + bytes_b + bytes_r + bytes_n + bytes_e; }
-};
-static ModGeom mod_geom(bool conjA, int M, int N, int K) {
-  ModGeom g;
-  g.Mr = conjA ? 2 * (int64_t)M : M;
-  g.Nr = 2 * (int64_t)N;
-  // the fewest tiles of at most 256 columns, all of the least width
-  g.gm = (int)((g.Mr + 255) / 256);
-  g.gn = (int)((g.Nr + 255) / 256);
-  g.bn = (int)round_up((g.Nr + g.gn - 1) / g.gn, 32);
-  g.Np = (int64_t)g.gn * g.bn;
-  const int per = conjA ? 1 : 2;  // real K per complex K
-  int64_t kmax = (int64_t)(kOzSliceCap / (2 * kMod)) / (g.Mr + g.Nr) / per;
-  kmax = std::max<int64_t>(kmax / 960 * 960, 960);
-  g.nseg = (int)((K + kmax - 1) / kmax);
-  g.kseg = (int)std::min<int64_t>(K, round_up((K + g.nseg - 1) / g.nseg, 64));
-  g.nseg = (K + g.kseg - 1) / g.kseg;
-  g.seg = round_up((int64_t)g.kseg * per, TC_BK);
-  g.kb = (int)(g.seg / TC_BK);
-  // K ranges: the count with the least modelled time, waves of pairs times a
-  // range's K blocks (0.26 us each at 256 columns) and about 4 us of epilogue, plus the
-  // residues written and read (nominal rates)
-  const int64_t items = (int64_t)g.gm * g.gn * kMod;
-  const int pairs = mod_pairs();
-  double best = 1e300;
-  g.gz = 1;
-  for (int z = 1; z <= std::min(32, std::max(1, g.kb / 4)); ++z) {
-    const double waves = (double)((items * z + pairs - 1) / pairs);
-    const double t = waves * ((g.kb + z - 1) / z * 1e-9 * g.bn + 4e-6) +
-                     z * 2.0 * kMod * (double)g.Mr * g.Nr / 6e12;
-    if (t < best) {
-      best = t;
-      g.gz = z;
-    }
-  }
-  g.kb_per = (g.kb + g.gz - 1) / g.gz;
-  g.gz = (g.kb + g.kb_per - 1) / g.kb_per;
-  g.nz = g.gz * g.nseg;
-  // blocks a row norm: about two waves of 256-thread blocks
-  const int rows_a = conjA ? M : (M + 255) / 256;
-  g.Sa = std::max(1, std::min({16, (1216 + rows_a - 1) / rows_a, (K + 31) / 32}));
-  g.Sb = std::max(1, std::min({16, (1216 + N - 1) / N, (K + 255) / 256}));
-  g.bytes_a = align256((size_t)kMod * g.Mr * g.seg * 2);
-  g.bytes_b = align256((size_t)kMod * g.Nr * g.seg * 2);
-  g.bytes_r = align256((size_t)g.nz * kMod * g.Mr * g.Np);
-  g.bytes_n = align256(((size_t)M * g.Sa + (size_t)N * g.Sb) * sizeof(int2));
-  g.bytes_e = align256(((size_t)M + N) * sizeof(int));
-  return g;
-}
-
-// Pieces of the larger output dimension, for products whose residues do not
-// fit the workspace even in the shortest K segments (or whose K is short: long
-// K segments keep the MMA pipeline full).  Every piece gives the bits of the
-// whole product.
-struct ModSplit {
-  bool split_m;
-  int piece;
-};
-static ModSplit mod_split(bool conjA, int M, int N, int K) {
-  ModSplit sp{M >= N, std::max(M, N)};
-  const int per = conjA ? 1 : 2;
-  const int64_t kreal = std::min<int64_t>((int64_t)K * per, 16384);
-  // real rows that fit with kreal columns, after the other operand's
-  const int64_t rows = (int64_t)(kOzSliceCap / (2 * kMod)) / std::max<int64_t>(kreal, 64);
-  const int64_t other = sp.split_m ? 2 * (int64_t)N : (conjA ? 2 * (int64_t)M : M);
-  const int64_t w = sp.split_m ? (conjA ? 2 : 1) : 2;  // real rows per row or column
-  const int64_t fit = std::max<int64_t>(1024, (rows - other) / w / 256 * 256);
-  if (fit < sp.piece) {
-    const int64_t np = (sp.piece + fit - 1) / fit;
-    sp.piece = (int)round_up((sp.piece + np - 1) / np, 128);
-  }
-  return sp;
-}
-
 void oz_reserve(System& s, bool conjA, int M, int N, int K) {
-  if (M <= 0 || N <= 0 || K <= 0) return;
-  const ModSplit sp = mod_split(conjA, M, N, K);
-  const int rest = (sp.split_m ? M : N) % sp.piece;  // the last piece may split K further
-  for (int piece : {std::min(sp.piece, sp.split_m ? M : N), rest})
-    if (piece > 0)
-      ensure(s.ws_oz, mod_geom(conjA, sp.split_m ? piece : M, sp.split_m ? N : piece, K).total());
+  if (M <= 0 || N <= 0 || K <= 0 || 8.0 * M * (double)N * K < kOzMinFlops) return;
+  ensure(s.ws_oz, mod_bound(conjA, M, N, K));
 }
 
 static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 alpha,
                           const double2* A, int64_t lda, const double2* B, int64_t ldb,
                           double2 beta, double2* C, int64_t ldc, cudaStream_t st,
                           const double* rowscale) {
-  const ModGeom g = mod_geom(conjA, M, N, K);
+  const ModGeom g = mod_geom(conjA, M, N, K, mod_pairs());
   ensure(s.ws_oz, g.total());
   char* base = s.ws_oz.p;
   __nv_bfloat16* pA = (__nv_bfloat16*)base;
@@ -933,7 +852,7 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
   // all moduli (2 Mr Nr Kr each)
   const double Kr = (double)g.seg * g.nseg;
   TimedScope ts(s, KF_GEMM_OZ, st, 2.0 * kMod * (double)g.Mr * g.Nr * Kr,
-                4.0 * kMod * ((double)g.Mr + g.Nr) * Kr + 2.0 * g.nz * kMod * (double)g.Mr * g.Nr);
+                4.0 * kMod * ((double)g.Mr + g.Nr) * Kr + 2.0 * g.gz * g.nseg * kMod * (double)g.Mr * g.Nr);
   if (conjA)
     k_mod_colnorm<<<dim3(M, g.Sa), 256, 0, st>>>(A, lda, K, na);
   else
@@ -972,7 +891,7 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
     a.gz = g.gz;
     a.kb_total = (int)(seg / TC_BK);
     a.kb_per = g.kb_per;
-    a.z0 = sgi * g.gz;
+    a.accum = sgi > 0;
     a.Np = g.Np;
     a.out = res;
     a.err = device_error_word(s);
@@ -990,12 +909,12 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
                                                                    : 2;
   const dim3 gc((M + 31) / 32, conjA ? (N + 15) / 16 : (N + 31) / 32);
   auto crt = [&](auto kernel) {
-    kernel<<<gc, 256, 0, st>>>(res, g.nz, M, N, g.Np, exa, exb, rowscale, o, C, ldc);
+    kernel<<<gc, 256, 0, st>>>(res, g.gz, M, N, g.Np, exa, exb, rowscale, o, C, ldc);
   };
   if (conjA)
-    g.nz > 1 ? crt(k_mod_crt<true, true>) : crt(k_mod_crt<true, false>);
+    g.gz > 1 ? crt(k_mod_crt<true, true>) : crt(k_mod_crt<true, false>);
   else
-    g.nz > 1 ? crt(k_mod_crt<false, true>) : crt(k_mod_crt<false, false>);
+    g.gz > 1 ? crt(k_mod_crt<false, true>) : crt(k_mod_crt<false, false>);
   PWH_LAUNCH_CHECK();
 }
 
@@ -1004,17 +923,12 @@ void oz_gemm(System& s, bool conjA, int M, int N, int K, double2 alpha, const do
              cudaStream_t st, const double* rowscale) {
   if (M <= 0 || N <= 0) return;
   const ModSplit sp = mod_split(conjA, M, N, K);
-  const int total = sp.split_m ? M : N;
-  for (int i0 = 0; i0 < total; i0 += sp.piece) {
-    const int n = std::min(sp.piece, total - i0);
-    if (sp.split_m)
-      // rows i0.. of C: columns i0.. of A (A^H) or rows i0.. of A
-      oz_gemm_piece(s, conjA, n, N, K, alpha, A + (conjA ? (int64_t)i0 * lda : (int64_t)i0), lda, B,
-                    ldb, beta, C + i0, ldc, st, rowscale ? rowscale + i0 : nullptr);
-    else
-      oz_gemm_piece(s, conjA, M, n, K, alpha, A, lda, B + (int64_t)i0 * ldb, ldb, beta,
-                    C + (int64_t)i0 * ldc, ldc, st, rowscale);
-  }
+  for (int64_t n0 = 0; n0 < N; n0 += sp.pn)
+    for (int64_t m0 = 0; m0 < M; m0 += sp.pm)
+      // rows m0.. of C: columns m0.. of A (A^H) or rows m0.. of A
+      oz_gemm_piece(s, conjA, (int)std::min<int64_t>(sp.pm, M - m0), (int)std::min<int64_t>(sp.pn, N - n0), K, alpha,
+                    A + (conjA ? m0 * lda : m0), lda, B + n0 * ldb, ldb, beta,
+                    C + n0 * ldc + m0, ldc, st, rowscale ? rowscale + m0 : nullptr);
 }
 
 }  // namespace pwh
