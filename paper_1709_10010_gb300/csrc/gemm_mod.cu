@@ -8,7 +8,10 @@
 //   exponent e with 2-norm <= 2^e over the whole K and becomes the integers
 //   X = round(x 2^(kT - e)), |X| <= 2^kT.  By Cauchy and Schwarz each real and
 //   imaginary part of the integer product is below 2^(2 kT) < P / 2, P the
-//   product of the moduli, so its residues determine it.  The only errors are
+//   product of the moduli, so its residues determine it.  In A^H B, whose real
+//   products keep real and imaginary parts apart, a column whose parts differ in norm
+//   by more than 2^kPartGap gets an exponent for each, so that the smaller keeps its
+//   bits; the real products then are rebuilt one by one.  The only errors are
 //   the rounding to X (relative to |a| |b|: 2^-kT, 62 bits) and the final
 //   FP64 rounding: no product of slices is dropped, and the exponents follow
 //   the rows' norms, not their largest elements.
@@ -36,6 +39,7 @@ namespace pwh {
 // ------------------------------------------------------------- the moduli ----
 constexpr int kT = 62;  // operands are integers of 2-norm at most 2^kT
 constexpr int kDigits = 6;
+constexpr int kPartGap = 4;
 struct ModTab {
   int p[kMod];
   // 2^16, 2^32 and 2^48 mod p, symmetric: the weights of X's 16-bit limbs
@@ -128,28 +132,34 @@ struct NormAcc {
   }
 };
 
-// Column j of X (K x J, ld) split over gridDim.y blocks: partial j gridDim.y + y.
+// Real and imaginary parts c of column j of X (K x J, ld) split over gridDim.y
+// blocks: partial (2 j + c) gridDim.y + y.
 __global__ void __launch_bounds__(256) k_mod_colnorm(const double2* __restrict__ X, int64_t ld, int K,
                                                      int2* __restrict__ part) {
-  __shared__ int2 red[8];
+  __shared__ int2 red[2][8];
   const int j = blockIdx.x;
   const double2* x = X + (size_t)j * ld;
-  NormAcc a;
+  NormAcc a[2];
   for (int k = blockIdx.y * 256 + threadIdx.x; k < K; k += gridDim.y * 256) {
     const double2 v = x[k];
-    a.add(v.x);
-    a.add(v.y);
+    a[0].add(v.x);
+    a[1].add(v.y);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const int E2 = __shfl_down_sync(0xffffffffu, a.E, o);
-    const float s2 = __shfl_down_sync(0xffffffffu, a.s, o);
-    a.merge(E2, s2);
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const int E2 = __shfl_down_sync(0xffffffffu, a[c].E, o);
+      const float s2 = __shfl_down_sync(0xffffffffu, a[c].s, o);
+      a[c].merge(E2, s2);
+    }
+    if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = make_int2(a[c].E, __float_as_int(a[c].s));
   }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_int2(a.E, __float_as_int(a.s));
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) a.merge(red[w].x, __int_as_float(red[w].y));
-    part[(size_t)j * gridDim.y + blockIdx.y] = make_int2(a.E, __float_as_int(a.s));
+  if (threadIdx.x < 2) {
+    const int c = threadIdx.x;
+    NormAcc t;
+    for (int w = 0; w < 8; ++w) t.merge(red[c][w].x, __int_as_float(red[c][w].y));
+    part[(2 * (size_t)j + c) * gridDim.y + blockIdx.y] = make_int2(t.E, __float_as_int(t.s));
   }
 }
 // Rows m of A (M x K, ld), columns split over gridDim.y blocks.
@@ -168,25 +178,41 @@ __global__ void __launch_bounds__(256) k_mod_rownorm(const double2* __restrict__
   }
   part[(size_t)m * gridDim.y + blockIdx.y] = make_int2(a.E, __float_as_int(a.s));
 }
-// e with norm <= 2^e from a row's partials, for the rows of both operands.
-__global__ void k_mod_exp(const int2* __restrict__ pa, int na, int Sa, const int2* __restrict__ pb,
-                          int nb, int Sb, int* __restrict__ ex) {
+// e with norm <= 2^e
+__device__ __forceinline__ int mod_exp(const NormAcc& a) {
+  if (a.E == 0x7ff) return kNonfinite;
+  if (!(a.s > 0.f)) return 0;
+  // s (1 + 1e-3) < 2^q covers the truncated fractions and the FP32 sum
+  int q;
+  frexpf(a.s * 1.001f, &q);
+  return a.E - 1023 + ((q + 1) >> 1);
+}
+// Exponents from the partials of the rows of A (na of them; parts = 1: one each)
+// and the columns of B (nb); parts = 2: two each, real and imaginary part, equal
+// (the norm of both) unless `apart` and the parts are further apart than kPartGap.
+__global__ void k_mod_exp(const int2* __restrict__ pa, int na, int Sa, int parts_a,
+                          const int2* __restrict__ pb, int nb, int Sb, bool apart,
+                          int* __restrict__ exa, int* __restrict__ exb) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= na + nb) return;
-  const int S = i < na ? Sa : Sb;
-  const int2* p = i < na ? pa + (size_t)i * Sa : pb + (size_t)(i - na) * Sb;
+  const int S = i < na ? Sa : Sb, parts = i < na ? parts_a : 2;
+  const int2* p = i < na ? pa + (size_t)i * S * parts : pb + (size_t)(i - na) * S * parts;
+  int* ex = i < na ? exa + (size_t)i * parts : exb + 2 * (size_t)(i - na);
   NormAcc a;
   for (int k = 0; k < S; ++k) a.merge(p[k].x, __int_as_float(p[k].y));
-  int e = 0;
-  if (a.E == 0x7ff) {
-    e = kNonfinite;
-  } else if (a.s > 0.f) {
-    // s (1 + 1e-3) < 2^q covers the truncated fractions and the FP32 sum
-    int q;
-    frexpf(a.s * 1.001f, &q);
-    e = a.E - 1023 + ((q + 1) >> 1);
+  if (parts == 1) {
+    ex[0] = mod_exp(a);
+    return;
   }
-  ex[i] = e;
+  NormAcc b;
+  for (int k = S; k < 2 * S; ++k) b.merge(p[k].x, __int_as_float(p[k].y));
+  const int e0 = mod_exp(a), e1 = mod_exp(b);
+  const bool two = apart && a.s > 0.f && b.s > 0.f && e0 != kNonfinite && e1 != kNonfinite &&
+                   abs(e0 - e1) > kPartGap;
+  a.merge(b.E, b.s);
+  const int e = mod_exp(a);
+  ex[0] = two ? e0 : e;
+  ex[1] = two ? e1 : e;
 }
 
 // ---------------------------------------------------------------- residues ----
@@ -250,13 +276,13 @@ __global__ void __launch_bounds__(256) k_mod_slice_cols(const double2* __restric
   const int k = 4 * (blockIdx.x * 256 + threadIdx.x);
   if (k >= seg) return;
   const double2* x = X + (size_t)j * ld;
-  const int e = ex[j];
+  const int er = ex[2 * j], ei = ex[2 * j + 1];
   float lr[4][4], li[4][4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const double2 v = k + u < K ? x[k + u] : make_double2(0.0, 0.0);
-    mod_limbs(v.x, e, lr[u]);
-    mod_limbs(v.y, e, li[u]);
+    mod_limbs(v.x, er, lr[u]);
+    mod_limbs(v.y, ei, li[u]);
   }
   char* o = (char*)(out + (size_t)(2 * j) * seg + k);
   each_mod<0>([&](auto I) {
@@ -315,7 +341,7 @@ __global__ void __launch_bounds__(256) k_mod_slice_b2(const double2* __restrict_
   const int k = blockIdx.x * 256 + threadIdx.x;
   if (2 * k >= seg) return;
   const double2 v = k < K ? B[(size_t)n * ld + k] : make_double2(0.0, 0.0);
-  const int e = ex[n];
+  const int e = ex[2 * n];
   float lr[4], li[4];
   mod_limbs(v.x, e, lr);
   mod_limbs(v.y, e, li);
@@ -699,7 +725,8 @@ __device__ __forceinline__ void crt_store(const CrtOut& o, double re, double im,
 
 // Complex (m, n) from the residues res[z][modulus][m'][n'].  op(A) = A^H: from
 // rows 2m, 2m+1 and columns 2n, 2n+1 (Re = C[2m][2n] + C[2m+1][2n+1], Im =
-// C[2m][2n+1] - C[2m+1][2n]); op(A) = A: (C[m][2n], C[m][2n+1]).  A block takes
+// C[2m][2n+1] - C[2m+1][2n], their residues added unless an operand's parts have
+// two exponents); op(A) = A: (C[m][2n], C[m][2n+1]).  A block takes
 // 32 m (a warp's lanes: coalesced C) by NB n, its residues through shared
 // memory (16-byte loads, all in flight; pitch of an odd number of words), those of
 // several K ranges (RANGES) added modulo p on the way (20,000 x 544 outputs: 0.24 ms; 530
@@ -782,16 +809,34 @@ __global__ void __launch_bounds__(256, 3)
     re[u].set(dr);
     im[u].set(di);
   }
-  const int ea = exa[m];
+  const int ea = exa[CONJ ? 2 * m : m], eai = CONJ ? exa[2 * m + 1] : ea;
   const double rs = rowscale ? rowscale[m] : 1.0;
 #pragma unroll
   for (int u = 0; u < 2 * PAIRS; ++u) {
     const int n = n0 + 2 * PAIRS * warp + u;
     if (n >= N) break;
-    const int eb = exb[n];
+    const int eb = exb[2 * n], ebi = exb[2 * n + 1];
     double x, y;
     if (ea == kNonfinite || eb == kNonfinite) {
       x = y = __longlong_as_double(0x7ff8000000000000ll);
+    } else if (CONJ && (ea != eai || eb != ebi)) {
+      // Re Re + Im Im and Re Im - Im Re
+      x = y = 0.0;
+#pragma unroll 1
+      for (int w = 0; w < 4; ++w) {
+        const bool ima = w & 1, imb = w == 1 || w == 2;
+        CrtDigits d;
+        each_mod<0>([&](auto I) {
+          constexpr int i = decltype(I)::value;
+          d.template add<i>(
+              (signed char)(mine[i * ROWS * PW + (ima ? PW : 0) + u / 2] >> (16 * (u & 1) + (imb ? 8 : 0))));
+        });
+        CrtFrac f;
+        f.set(d);
+        const double v = f.value(ima ? eai : ea, imb ? ebi : eb);
+        if (w < 2) x += v;
+        else y += w == 2 ? v : -v;
+      }
     } else {
       x = re[u].value(ea, eb);
       y = im[u].value(ea, eb);
@@ -845,9 +890,10 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
   __nv_bfloat16* pB = (__nv_bfloat16*)(base + g.bytes_a);
   unsigned char* res = (unsigned char*)(base + g.bytes_a + g.bytes_b);
   int2* na = (int2*)(base + g.bytes_a + g.bytes_b + g.bytes_r);
-  int2* nb = na + (size_t)M * g.Sa;
+  const int parts = conjA ? 2 : 1;  // exponents of a row of op(A)
+  int2* nb = na + (size_t)M * g.Sa * parts;
   int* exa = (int*)((char*)na + g.bytes_n);
-  int* exb = exa + M;
+  int* exb = exa + (size_t)M * parts;
   // timed as its own family: the work is the real BF16 tensor-core GEMMs of
   // all moduli (2 Mr Nr Kr each)
   const double Kr = (double)g.seg * g.nseg;
@@ -860,7 +906,7 @@ static void oz_gemm_piece(System& s, bool conjA, int M, int N, int K, double2 al
   PWH_LAUNCH_CHECK();
   k_mod_colnorm<<<dim3(N, g.Sb), 256, 0, st>>>(B, ldb, K, nb);
   PWH_LAUNCH_CHECK();
-  k_mod_exp<<<(M + N + 255) / 256, 256, 0, st>>>(na, M, g.Sa, nb, N, g.Sb, exa);
+  k_mod_exp<<<(M + N + 255) / 256, 256, 0, st>>>(na, M, g.Sa, parts, nb, N, g.Sb, conjA, exa, exb);
   PWH_LAUNCH_CHECK();
   for (int sgi = 0; sgi < g.nseg; ++sgi) {
     const int k0 = sgi * g.kseg, kk = std::min(g.kseg, K - k0);

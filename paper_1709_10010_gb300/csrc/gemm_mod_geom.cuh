@@ -85,8 +85,10 @@ inline ModGeom mod_geom(bool conjA, int M, int N, int K, int pairs) {
   g.bytes_a = oz_align((size_t)kMod * g.Mr * g.seg * 2);
   g.bytes_b = oz_align((size_t)kMod * g.Nr * g.seg * 2);
   g.bytes_r = oz_align(g.gz * plane);
-  g.bytes_n = oz_align(((size_t)M * g.Sa + (size_t)N * g.Sb) * 8);
-  g.bytes_e = oz_align(((size_t)M + N) * 4);
+  // norms and exponents: one of a row of A, two of a column
+  const size_t pa = conjA ? 2 : 1;
+  g.bytes_n = oz_align(((size_t)M * g.Sa * pa + (size_t)N * g.Sb * 2) * 8);
+  g.bytes_e = oz_align((M * pa + 2 * (size_t)N) * 4);
   return g;
 }
 
@@ -131,7 +133,7 @@ inline size_t mod_bound(bool conjA, int M, int N, int K) {
   const size_t residues = std::min(kOzResidueCap, plane > kOzResidueCap ? kOzResidueCap : plane * ranges);
   // rows of a piece: their operand residues over 64 of K fit
   const size_t rows = std::min<size_t>((size_t)M + N, kOzOperandCap / (2 * kMod * 64) + 256);
-  return operands + residues + rows * (16 * 8 + 4) + 5 * 256;
+  return operands + residues + rows * 2 * (16 * 8 + 4) + 5 * 256;
 }
 
 }  // namespace pwh
