@@ -32,6 +32,7 @@
 #include "common.cuh"
 #include "gemm.cuh"
 #include "gemm_mod_geom.cuh"
+#include "pair_ring.cuh"
 #include "tc_ptx.cuh"
 
 namespace pwh {
@@ -424,6 +425,12 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
       "h"((uint16_t)3)
       : "memory");
 }
+// arrive on this CTA's mbarrier once the MMAs issued so far are done
+__device__ __forceinline__ void mma_commit_pair_own(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                   su32(bar))
+               : "memory");
+}
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -437,8 +444,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   uint64_t* empty = full + kPairStages;
   uint64_t* tfull = empty + kPairStages;  // [2]
   uint64_t* tempty = tfull + 2;           // [2], CTA 0's is used
-  uint32_t* tmem_slot = (uint32_t*)(tempty + 2);
+  uint64_t* quiet = tempty + 2;           // CTA 0's: the MMAs after a time-out are done
+  uint32_t* tmem_slot = (uint32_t*)(quiet + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  volatile int* fills1 = abort_flag + 1;  // CTA 0's: slots that CTA 1 filled
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
@@ -454,6 +463,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], 16);  // eight epilogue warps in each CTA
     }
+    mbar_init(quiet, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -535,6 +545,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         if (ok) mma_commit_pair(&tfull[buf]);
       }
     }
+    if (!ok) {
+      // no epilogue waits for the last MMAs: they read shared and write tensor memory
+      mma_commit_pair_own(quiet);
+      mbar_wait(quiet, 0, nullptr);
+    }
   } else if (warp < 8) {
     const int sub = warp & 3, half = warp >> 2;
     // columns of this warp: the first 128 of the tile or the others
@@ -614,10 +629,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     }
   }
   __syncwarp();
-  // CTA 0's producer: every copy of the pair that was announced has landed
-  // before shared memory goes away (its barrier counts both CTAs' bytes)
-  if (warp == 8 && lane == 0 && rank == 0) {
+  // Shared memory goes away only after everything that comes in from outside the
+  // thread has landed.  Each producer: the MMA issuer's releases of its last slots (none
+  // come after a time-out, the flag then ends the wait).  CTA 0's: the copies of both
+  // CTAs, whose counts differ after a time-out (pair_drain).
+  if (warp == 8 && lane == 0) {
     for (int j = max(0, issued - kPairStages); j < issued; ++j)
+      if (!mbar_wait(&empty[j % kPairStages], (j / kPairStages) & 1, abort_flag)) break;
+    if (rank == 1)
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta0(su32((const void*)fills1))),
+                   "r"(issued)
+                   : "memory");
+  }
+  __syncwarp();
+  pair_sync();
+  if (warp == 8 && lane == 0 && rank == 0) {
+    const PairDrain d = pair_drain(issued, *fills1, kPairStages);
+    const int bytes = kPairABytes + (args.bn / 2) * TC_BK * 2;  // one CTA's loads
+    for (int j = d.arm0; j < d.arm1; ++j) mbar_expect_tx(&full[j % kPairStages], bytes);
+    for (int j = d.wait0; j < d.wait1; ++j)
       mbar_wait(&full[j % kPairStages], (j / kPairStages) & 1, nullptr);
   }
   tc_fence_before();
