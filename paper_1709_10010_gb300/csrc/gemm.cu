@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256) k_splitk_reduce_wide(int M, int N, int ns
 // Tile shapes (BM, BN, TM, TN, BK) by the width N of the product: narrow
 // products (a few unconverged bands) take tall thin tiles so that no
 // arithmetic is spent on padding columns; FP32 takes 8 x 8 (or 8 x 4)
-// outputs per thread, FP64 by plan64 (its pipe, not shared memory, is the
+// outputs per thread, FP64 by plan64 (gemm_plan.cuh; its pipe, not shared memory, is the
 // limit).
 template <typename TS, typename T, int BM, int BN, int TM, int TN, int BK>
 static void cgemm_launch(System& s, bool conjA, int M, int N, int K, cx<TS> alpha, const cx<TS>* A,
@@ -258,39 +258,6 @@ static void cgemm_launch(System& s, bool conjA, int M, int N, int K, cx<TS> alph
   }
 }
 
-// Tile and split-K of an FP64 product on the FP64 pipe: the least modelled
-// clocks, waves of blocks over 152 SMs times a block's multiply-adds (four a
-// complex pair at the measured 1.6 a clock of an SM) and 1,200 clocks of latency,
-// plus the reduction of the partials.  A tile much larger than the product
-// computes padding, and few tiles leave the pipe of most SMs idle: 32 x 16 over
-// K = 1503 took 176 us in 256 x 16 tiles and takes 20, 1503 x 16 over K = 32 139 us
-// on six of them and takes 14, 256^3 143 us and takes 45 (oz_gemm).
-struct Plan64 {
-  int shape, split;
-  double us;  // modelled time
-};
-constexpr int kShape64[7][2] = {{64, 64}, {128, 32}, {256, 16}, {256, 8}, {32, 32}, {32, 16}, {16, 16}};
-static Plan64 plan64(int M, int N, int K, bool part) {
-  Plan64 best{0, 1, 1e300};
-  for (int i = 0; i < 7; ++i) {
-    const int BM = kShape64[i][0], BN = kShape64[i][1];
-    const int64_t tiles = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-    for (int w = 0; w <= 6; ++w) {
-      int split = w == 0 ? 1 : (int)((152 * (int64_t)w + tiles - 1) / tiles);
-      split = std::max(1, std::min(split, std::min(256, K / 16)));
-      if ((double)split * M * N * 16.0 > 64.0 * (1 << 20)) continue;
-      const int chunk = (((K + split - 1) / split) + 15) / 16 * 16;
-      split = std::max(1, (K + chunk - 1) / std::max(chunk, 1));
-      const double waves = (double)((tiles * split + 151) / 152);
-      double clk = waves * (2.5 * BM * BN * chunk + 1200.0);
-      if (split > 1 || part) clk += 5000.0 + split * (double)M * N * 32.0 / 3000.0;
-      if (clk < best.us) best = {i, split, clk};
-    }
-  }
-  best.us /= 2000.0;  // 2 GHz
-  return best;
-}
-
 template <typename TS, typename T>
 static void cgemm_impl(System& s, bool conjA, int M, int N, int K, cx<TS> alpha, const cx<TS>* A,
                        int64_t lda, const cx<TS>* B, int64_t ldb, cx<TS> beta, cx<TS>* C,
@@ -326,18 +293,6 @@ static void cgemm_impl(System& s, bool conjA, int M, int N, int K, cx<TS> alpha,
       default: run(I<16>{}, I<16>{}, I<1>{}, I<1>{}, I<16>{}); break;
     }
   }
-}
-
-// Whether an FP64 product goes to the tensor cores (oz_gemm): at least
-// kOzMinFlops, and the modelled time there is the smaller: about 40 us of launches
-// and latency, the operands read twice and written as 64 bytes a complex number
-// (5 TB/s), 128 tensor operations a complex multiply-add (1.2 PFLOP/s).  Products
-// of a few columns stay on the FP64 pipe whatever their length.
-static bool oz_wins(int M, int N, int K) {
-  if (8.0 * M * (double)N * K < kOzMinFlops) return false;
-  const double oz = 40.0 + ((double)M + N) * K * 96.0 / 5e6 + 128.0 * M * (double)N * K / 1.2e9 +
-                    (double)M * N * 80.0 / 3e6;
-  return oz < plan64(M, N, K, false).us;
 }
 
 // The sliced tensor-core paths launch one block row per column of A (A^H B)

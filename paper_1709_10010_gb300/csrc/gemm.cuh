@@ -1,6 +1,7 @@
 // Internal GEMM launchers of libpwh.
 #pragma once
 #include "common.cuh"
+#include "gemm_plan.cuh"
 
 namespace pwh {
 
@@ -29,10 +30,6 @@ void cgemm_f32_simt(System& s, bool conjA, int M, int N, int K, double2 alpha, c
 // Grow the residue workspace for op(A) B of these sizes now (so that
 // later products of at most this size allocate nothing).
 void oz_reserve(System& s, bool conjA, int M, int N, int K);
-// Products of at least this many flops (8 M N K) may take oz_gemm in
-// cgemm<double> (where its modelled time is the smaller, gemm.cu).
-constexpr double kOzMinFlops = 2e7;
-
 // FP64-equivalent complex GEMM on the BF16 tensor cores (gemm_mod.cu): same
 // contract as cgemm<double>, results within FP64-level rounding (62-bit
 // integers, exact products by residues); a row of op(A) or column of B with an
