@@ -120,9 +120,10 @@ struct JacobiArgsT {
   double tol;
   int* out_buf;   // buffer index (0/1) holding the result, sweeps used
   int* conv;      // per-sweep convergence flag written by block 0
-  const int* skip;  // optional device word: nonzero = already diagonal, no sweep
-  // optional device word: max |A_ii|; pairs with |A_pq| <= 1e-15 of it keep
-  // their element and are not rotated (FP64 only)
+  // of a polish (KEEP), else null.  skip: nonzero = already diagonal, no sweep;
+  // dmax: max |A_ii|, pairs with |A_pq| <= 1e-15 of it keep their element and are not
+  // rotated
+  const int* skip;
   const unsigned long long* dmax;
   GridBar gb;
 };
@@ -138,7 +139,8 @@ __device__ __forceinline__ void cluster_sync_all() {
 // CLUSTER: the grid is one thread-block cluster and rounds are separated by
 // the hardware cluster barrier; otherwise by the bounded grid barrier of a
 // cooperative launch.
-template <typename T, bool CLUSTER>
+// KEEP (FP64): the polish of an almost diagonal matrix, with a.dmax.
+template <typename T, bool CLUSTER, bool KEEP = false>
 __global__ void k_jacobi(JacobiArgsT<T> a) {
   extern __shared__ __align__(16) unsigned char jsm[];
   const int n = a.n, np = a.np, P = np / 2;
@@ -151,9 +153,9 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
   const int nth = gridDim.x * blockDim.x;
   unsigned epoch = 0;  // grid barriers passed
   int cur = 0, sweep = 0;
-  const int max_sweeps = a.skip && *a.skip ? 0 : a.max_sweeps;
+  const int max_sweeps = KEEP && *a.skip ? 0 : a.max_sweeps;
   double keep2 = -1.0;  // |A_pq|^2 up to which a pair is left alone
-  if (sizeof(T) == 8 && a.dmax) {
+  if constexpr (KEEP) {
     const double d = 1e-15 * __longlong_as_double((long long)*a.dmax);
     keep2 = d * d;
   }
@@ -167,7 +169,7 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
         cx<T> sv = mk<T>(0, 0);
         if (q < n) {
           const cx<T> apq = A[(size_t)q * n + p];
-          if (sizeof(T) == 4 || !((double)apq.x * apq.x + (double)apq.y * apq.y <= keep2))
+          if (!KEEP || !((double)apq.x * apq.x + (double)apq.y * apq.y <= keep2))
             jacobi_rotation<T>(apq, A[(size_t)p * n + p].x, A[(size_t)q * n + q].x, c, sv);
         }
         pp[k] = p;
@@ -197,7 +199,7 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
           cx<T> y00, y01, y10, y11;
           // neither pair rotates (the polish of an almost diagonal matrix):
           // the block moves to the other buffer without FP64 arithmetic
-          const bool still = sizeof(T) == 8 && keep2 >= 0 && ck == (T)1 && cl == (T)1 &&
+          const bool still = KEEP && ck == (T)1 && cl == (T)1 &&
                              sk.x == (T)0 && sk.y == (T)0 && sl.x == (T)0 && sl.y == (T)0;
           if (still) {
             y00 = a00; y01 = a01; y10 = a10; y11 = a11;
@@ -236,7 +238,7 @@ __global__ void k_jacobi(JacobiArgsT<T> a) {
           const T cl = crot[l];
           const cx<T> sl = srot[l];
           const cx<T> q0 = Qc[(size_t)pl * n + i];
-          if (sizeof(T) == 8 && keep2 >= 0 && ql < n && cl == (T)1 && sl.x == (T)0 && sl.y == (T)0) {
+          if (KEEP && ql < n && cl == (T)1 && sl.x == (T)0 && sl.y == (T)0) {
             Qn[(size_t)pl * n + i] = q0;
             Qn[(size_t)ql * n + i] = Qc[(size_t)ql * n + i];
           } else if (ql < n) {
@@ -1461,6 +1463,8 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
   static int cluster_size = 0;  // largest cluster (16 or 8) that fits, 0 if none
   std::call_once(attr_once, [] {
     cudaFuncSetAttribute(k_jacobi<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if constexpr (sizeof(T) == 8)
+      cudaFuncSetAttribute(k_jacobi<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_jacobi<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_jacobi<T, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int cs : {16, 8}) {
@@ -1506,7 +1510,10 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
   int dev = 0, nsm = 0, per_sm = 0;
   PWH_CUDA(cudaGetDevice(&dev));
   PWH_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  PWH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi<T, false>, 256, smem));
+  const void* kernel = (const void*)k_jacobi<T, false>;
+  if constexpr (sizeof(T) == 8)
+    if (skip) kernel = (const void*)k_jacobi<T, false, true>;
+  PWH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem));
   // FP32 stage: few blocks (the per-round barrier latency dominates);
   // FP64 stage: every SM, the FP64 units are the limit
   const int64_t items = (int64_t)P * P + (int64_t)n * P;
@@ -1514,7 +1521,7 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
   const int want = (int)std::max<int64_t>(1, std::min<int64_t>((items + per_block - 1) / per_block, nsm));
   const int blocks = std::max(1, std::min(want, nsm * std::max(per_sm, 1)));
   void* args[] = {&a};
-  PWH_CUDA(cudaLaunchCooperativeKernel((void*)k_jacobi<T, false>, blocks, 256, args, smem, st));
+  PWH_CUDA(cudaLaunchCooperativeKernel(kernel, blocks, 256, args, smem, st));
   note_launch();
 }
 
