@@ -1772,6 +1772,41 @@ __global__ void __launch_bounds__(128) k_refine_m(double2* __restrict__ S,
   }
 }
 
+// ---- range of the matrix -------------------------------------------------------
+// FP32 sweeps square elements down to 1e-7 of the largest: below about 1e-19 they
+// vanish and nothing rotates, and a sweep in FP32 pairs that has to turn vectors by
+// large angles leaves them unitary to 1e-6 only (eigenvalues off by 1e-12 at a scale
+// of 1e-30).  A matrix whose largest element lies outside [2^-20, 2^41) is scaled by
+// a power of two, exactly, to one near 1; the others keep their bits.
+__device__ __forceinline__ int eig_exponent(const unsigned* mx) {
+  const int eb = (int)(*mx >> 20);  // biased exponent of the largest |Re|, |Im|
+  return eb == 0x7ff || *mx == 0 || (eb >= 1023 - 20 && eb <= 1023 + 40) ? 0 : eb - 1023;
+}
+__global__ void __launch_bounds__(256) k_eig_max(const double2* __restrict__ H, int64_t ldh, int n,
+                                                 unsigned* __restrict__ mx) {
+  unsigned m = 0;
+  for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < (int64_t)n * n; t += gridDim.x * 256ll) {
+    const double2 v = H[(t / n) * ldh + t % n];
+    m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(mx, m);
+}
+__global__ void __launch_bounds__(256) k_eig_scale(const double2* __restrict__ H, int64_t ldh, int n,
+                                                   const unsigned* __restrict__ mx,
+                                                   double2* __restrict__ out) {
+  const int e = eig_exponent(mx);
+  for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < (int64_t)n * n; t += gridDim.x * 256ll) {
+    double2 v = H[(t / n) * ldh + t % n];
+    if (e) v = make_double2(scalbn(v.x, -e), scalbn(v.y, -e));
+    out[t] = v;
+  }
+}
+__global__ void k_eig_unscale(double* __restrict__ d, int n, const unsigned* __restrict__ mx) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, e = eig_exponent(mx);
+  if (i < n && e) d[i] = scalbn(d[i], e);
+}
+
 // ---- the first FP64 sweep in FP32 pairs ---------------------------------------
 // One cyclic sweep (the rounds and rotations of k_jacobi<double>) on the almost
 // diagonal A: its diagonal in FP64, off-diagonal elements and Q as pairs hi + lo of
@@ -2002,9 +2037,9 @@ static void pair_sweep(System& s, DenseWs& w, double2* A, double2* A1, double2* 
 }
 
 static size_t jacobi_ws_bytes(size_t nn, int n) {
-  // FP64: A0, A1, Q0, Q1, G;  FP32: a0, a1, q0, q1;  diagonal d;  the
-  // refinement's per-index arrays
-  return 5 * nn * sizeof(double2) + 4 * nn * sizeof(float2) + (size_t)n * sizeof(double) + 512 +
+  // FP64: A0, A1, Q0, Q1, G, the scaled matrix;  FP32: a0, a1, q0, q1;  diagonal d;
+  // the refinement's per-index arrays
+  return 6 * nn * sizeof(double2) + 4 * nn * sizeof(float2) + (size_t)n * sizeof(double) + 512 +
          refine_bytes(n);
 }
 
@@ -2019,7 +2054,8 @@ void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, in
   double2* Q0 = A1 + nn;
   double2* Q1 = Q0 + nn;
   double2* G = Q1 + nn;
-  float2* a0 = (float2*)(G + nn);
+  double2* Hs = G + nn;
+  float2* a0 = (float2*)(Hs + nn);
   float2* a1 = a0 + nn;
   float2* q0 = a1 + nn;
   float2* q1 = q0 + nn;
@@ -2032,12 +2068,24 @@ void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, in
   //   4-6   FP32 stage: result buffer index, sweeps, rounds logged
   //   8-9   FP64 stage: result buffer index, sweeps
   //   12    convergence flag of the grid-wide kernel (launch_jacobi)
+  //   13    largest element, where the matrix is scaled (eig_exponent)
   int* out_buf = (int*)(ctl + 8);
   int* ob32 = (int*)(ctl + 4);
   const int gq = (int)std::min<int64_t>(1024, ((int64_t)nn + 255) / 256);
   const double2 one = make_double2(1, 0), zero = make_double2(0, 0);
   const bool warm = warm_m0 > 0 && Qkeep;
   double2* Q = Q0;
+  // The first FP64 sweep in FP32 pairs needs the FP32 stage's basis, so the matrix
+  // comes in a range where that works.
+  const bool scaled = polish && n >= kRefineMinN;
+  if (scaled) {
+    k_eig_max<<<gq, 256, 0, st>>>(H, ldh, n, ctl + 13);
+    PWH_LAUNCH_CHECK();
+    k_eig_scale<<<gq, 256, 0, st>>>(H, ldh, n, ctl + 13, Hs);
+    PWH_LAUNCH_CHECK();
+    H = Hs;
+    ldh = n;
+  }
   {
     TimedScope ts(s, KF_JACOBI32, st);
     // ---- stage 1 (FP32): rotate the start to near-diagonal
@@ -2191,6 +2239,10 @@ void jacobi_eigh(System& s, DenseWs& w, const double2* H, int64_t ldh, int n, in
   }
   k_diag_of<double><<<(n + 255) / 256, 256, 0, st>>>(A0, A1, out_buf, n, dg);
   PWH_LAUNCH_CHECK();
+  if (scaled) {
+    k_eig_unscale<<<(n + 255) / 256, 256, 0, st>>>(dg, n, ctl + 13);
+    PWH_LAUNCH_CHECK();
+  }
   k_select_buf64<<<gq, 256, 0, st>>>(Q0, Q1, out_buf, (int64_t)nn, G);
   PWH_LAUNCH_CHECK();
   const int sb = (int)std::min<int64_t>(64, ((int64_t)nn + 1023) / 1024);
