@@ -580,12 +580,22 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
 // one of 512 from 96 on, where the columns fill the SM's shared memory (64 bands,
 // blocks of 256 and 512: 40 152 and 187 us, 72 1.12 and 1.42 ms, 90 2.13 and 2.28,
 // 96 3.67 and 3.28, 120 6.43 and 5.79, 144 15.4 and 14.1).  FP32 waits for shared
-// memory: 256 threads, two blocks an SM by shared
-// memory, at 90^3 (0.461 ms for 128 bands, 0.470 with 512); one block of 1,024 where
-// the columns leave room for one (144^3, 512 bands: 8.28 ms, 8.43 with 512, 9.8 with
-// 768).
+// memory: two blocks of 256 an SM where they fit, larger blocks where the columns
+// leave room for one (128 bands, blocks of 256 / 512 / 1,024: 30 25 / 30 / 75 us, 48 68 /
+// 94 / 143, 60 135 / 174 / 244, 72 231 / 261 / 348, 90 494 / 505 / 617, 96 558 / 572 /
+// 709, 120 1.28 / 1.23 / 1.36 ms, 144 2.70 / 2.26 / 2.15).
 template <typename T, int N>
-constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 120 ? 1024 : 256) : (N >= 96 ? 512 : 256);
+constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 144 ? 1024 : N >= 120 ? 512 : 256)
+                                                            : (N >= 96 ? 512 : 256);
+// FP32 where a launch has at most kFewPlanes blocks, about two an SM, so that a
+// block's own latency is the pass: 512 threads (one band, 256 / 512: 60 10.7 / 10.2 us,
+// 80 14.2 / 12.2, 90 15.7 / 13.8; four bands, 72 15.4 / 14.2, 90 28.6 / 26.0; below 48
+// no difference).
+constexpr int kFewPlanes = 360;
+template <typename T, int N>
+constexpr int plane_threads_few =
+    std::is_same<T, float>::value && N >= 48 && N < 144 ? 512 : plane_threads<T, N>;
+template <int NT> using Threads = std::integral_constant<int, NT>;
 
 // Shared memory of the plane pass for `rows` rows per chunk.
 template <typename T, int N> constexpr size_t ks_plane_smem(int ncols, int rows) {
@@ -721,6 +731,8 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
   std::call_once(once, [] {
     cudaFuncSetAttribute(ks_zinv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaFuncSetAttribute(ks_plane<T, N, plane_threads<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(ks_plane<T, N, plane_threads_few<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         227 * 1024);
     cudaFuncSetAttribute(ks_zfwd<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   });
   const cx<T>* tw = (const cx<T>*)a.tw;
@@ -733,11 +745,17 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
                                                  s.d_perm, W, a.wband, a.spb);
       break;
     case SPEC_PLANE: {
-      constexpr int NT = plane_threads<T, N>;
       const int rows = plane_rows<T, N>(s, a);
-      ks_plane<T, N, NT><<<dim3(N, a.bb), NT, ks_plane_smem<T, N>(s.ncols, rows), a.st>>>(
-          W, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V, s.plan[0].tw_off,
-          tw, rows);
+      auto run = [&](auto nt) {
+        constexpr int NT = decltype(nt)::value;
+        ks_plane<T, N, NT><<<dim3(N, a.bb), NT, ks_plane_smem<T, N>(s.ncols, rows), a.st>>>(
+            W, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V, s.plan[0].tw_off,
+            tw, rows);
+      };
+      if (N * a.bb <= kFewPlanes)
+        run(Threads<plane_threads_few<T, N>>{});
+      else
+        run(Threads<plane_threads<T, N>>{});
       break;
     }
     case SPEC_ZFWD:
