@@ -13,22 +13,24 @@
 namespace pwh {
 
 // dst[b][i] = src[b][idx[i]]: bands between the public and the internal order,
-// both ways as gathers (idx = int_to_pub or pub_to_int).  Bound by L2: a block takes
-// a run of one band, whose 16-byte reads stay within the band (scattered 16-byte
-// writes filled half a sector each: the way out took 1.40 ms for 512 bands of
-// 161,235 plane waves and takes 0.46 as a gather).
+// both ways as gathers (idx = int_to_pub or pub_to_int).  Bound by L2: neighbouring
+// threads take neighbouring elements of one band, whose 16-byte reads stay within
+// the band (scattered 16-byte writes filled half a sector each: the way out took
+// 1.40 ms for 512 bands of 161,235 plane waves and takes 0.46 as a gather).  One
+// range over all bands, so that few short bands fill their blocks (30^3, 2 to 12
+// bands: H 24.7 us, with a row of blocks a band 25.7 to 26.8).
 __global__ void __launch_bounds__(256) k_permute(const double2* __restrict__ src, int64_t lds, int64_t npw,
                                                  int nb, const int32_t* __restrict__ idx,
                                                  double2* __restrict__ dst, int64_t ldd) {
-  const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
-  if (i >= npw) return;
-  const int64_t j = idx[i];
-  for (int b = blockIdx.y; b < nb; b += gridDim.y) dst[b * ldd + i] = src[b * lds + j];
+  const int64_t tot = npw * nb;
+  for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < tot; t += gridDim.x * (int64_t)256) {
+    const int64_t b = t / npw, i = t - b * npw;
+    dst[b * ldd + i] = src[b * lds + idx[i]];
+  }
 }
 
-static dim3 permute_grid(int64_t npw, int nb) {
-  // four bands a thread where there are many (the index is read once for them)
-  return dim3((unsigned)((npw + 255) / 256), (unsigned)std::min(65535, nb > 64 ? (nb + 3) / 4 : nb));
+static int permute_grid(int64_t npw, int nb) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(152 * 16, (npw * nb + 255) / 256));
 }
 
 void permute_public_to_internal(System& s, const double2* src, double2* dst, int nb, int64_t lds) {
