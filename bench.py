@@ -613,12 +613,12 @@ def run_batched(pwh, syn, torch, ncells=32, nthreads=16):
 
 # The FP64-accurate FFT passes of the compiled box sizes run in double-float
 # arithmetic (pairs of FP32 numbers) on the FP32 pipes: a double-float sum is
-# 11 FP32 instructions, a complex product 40, and the nominal 5 N log2 N flops
+# 17 FP32 instructions, a complex product 38, and the nominal 5 N log2 N flops
 # of a radix-2 butterfly are one complex product and two complex sums in 10, so
-# one FP64-equivalent flop costs 8.4 FP32 instructions (transforms with fewer
+# one FP64-equivalent flop costs 10.6 FP32 instructions (transforms with fewer
 # products than nominal can pass this rate); the pipes issue 152 x 128 x 2.07e9
 # of those a second (half the FP32 flop rate, which counts an FMA as two).
-DF_FP32_OPS_PER_FLOP = (40 + 4 * 11) / 10
+DF_FP32_OPS_PER_FLOP = (38 + 4 * 17) / 10
 DF_ALU_TFLOPS = FP32_ALU_TFLOPS / 2 / DF_FP32_OPS_PER_FLOP
 
 FAMILY_BOUND = {
@@ -673,7 +673,7 @@ def family_roofline(fam, d, s=None):
         achieved = work / sec / 1e12
     elif key == "df":
         peak, unit = DF_ALU_TFLOPS, "TFLOP/s"
-        psrc = "derived double-float rate (FP32 instruction rate / 8.4)"
+        psrc = "derived double-float rate (FP32 instruction rate / 10.6)"
         achieved = work / sec / 1e12
     elif key is None:
         peak, unit = None, "TFLOP/s"

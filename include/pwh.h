@@ -57,9 +57,10 @@ typedef enum {
                          the FFT passes of the compiled cubic boxes (edges 30,
                          36, 40, 48, 50, 60, 72, 80, 90, 96, 120, 144), which
                          compute in double-float (pairs of FP32 numbers, 48
-                         significant bits, about 2^-46 relative rounding per
-                         operation), and the large GEMMs (62-bit integers, exact
-                         products by residues on the tensor cores) */
+                         significant bits; relative rounding of a sum below 2^-45,
+                         of a sum of products relative to the products), and
+                         the large GEMMs (62-bit integers, exact products by
+                         residues on the tensor cores) */
   PWH_MIXED = 1,      /* FFT + potential in FP32; projector GEMMs on the BF16
                          tensor cores with FP32 accumulation, each operand split
                          into two BF16 terms (hi*hi + hi*lo + lo*hi, about 16
@@ -518,8 +519,12 @@ pwh_status pwh_subspace_cholqr(pwh_system* sys, int32_t precision, int32_t k, co
  * uses it: C = alpha op(A) B + beta C, op(A) = A^H when conj_a else A; op(A)
  * is M x K, B is K x N, C is M x N; all DEVICE complex128, column-major with
  * the given leading dimensions (lda >= rows of A as stored).  alpha, beta:
- * HOST double[2] (re, im).  precision PWH_FP64: FP64 arithmetic (large
- * products as exact integer products by residues on the tensor cores);
+ * HOST double[2] (re, im).  precision PWH_FP64: FP64 arithmetic; products of
+ * at least 2e8 flops (8 M N K), where that is modelled faster, as exact
+ * products of integers on the tensor cores, 62 bits of the 2-norm of each row
+ * of op(A) and column of B (of its real and imaginary part in A^H B when
+ * these differ), an error of about sqrt(2 K) 2^-60 of the product of the two
+ * norms; a row or column with an infinity or NaN gives NaN;
  * PWH_MIXED: operands rounded to FP32, FP32 accumulation (relative error about
  * sqrt(K) 1e-7), result widened (products of at least 4e8 flops and 48
  * columns of A^H B or 96 of A B, or 1 and 16 columns when K (A^H B) or M (A B)

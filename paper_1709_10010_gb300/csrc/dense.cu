@@ -1541,12 +1541,12 @@ static void launch_jacobi(System& s, DenseWs& w, cx<T>* A0, cx<T>* A1, cx<T>* Q0
 // them (k_jacobi_pair_sweep), against two to three (30 in large clusters) sweeps
 // of n - 1 grid-wide rounds on the FP64 pipe (60 us a round at n = 1088).  The
 // whole FP64 eigensolve, FP32 stage included: n = 1088 137 -> 42 ms, 1632 587 ->
-// 126, 408 21.7 -> 14.0, 256 10.4 -> 8.3, five 128-fold levels 311 -> 31;
+// 126, 408 21.7 -> 14.0, 256 (random) 16.2 -> 15.3, five 128-fold levels 311 -> 31;
 // eigenvectors orthonormal to 3e-15 instead of 1e-13.  Without the first sweep (three
 // refinement steps from the FP32 basis) n = 1088 takes 20 ms to the same
 // accuracy, but with eigenvector phases that differ by 1e-6 from the cyclic
-// sweeps'.  Below kRefineMinN the products run on the FP64 pipe and gain
-// nothing.
+// sweeps'.  At kRefineMinN the FP64 stage takes 5.1 ms (its products, below 2e8 flops,
+// on the FP64 pipe) against 5.9 of the sweeps; smaller matrices gain less.
 constexpr int kRefineMinN = 256;
 struct RefineWs {
   double* dS;              // S_ii
@@ -1666,7 +1666,8 @@ __global__ void __launch_bounds__(128) k_refine_best(const double2* __restrict__
     atomicMax(&w.mx[0], (unsigned long long)__double_as_longlong(mg));
   }
 }
-// Pair rotations; done = max |F_ij| <= tol max |F_ii| (a NaN is not done).
+// Pair rotations; done = max |F_ij| <= tol max |F_ii|.  (The maxima pass over NaN: a
+// matrix of NaN counts as done, no sweep could mend it, and its results are NaN.)
 __global__ void k_refine_pairs(const double2* __restrict__ S, const double2* __restrict__ Gm, int n,
                                double lim, double tol, RefineWs w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1820,7 +1821,8 @@ __global__ void k_eig_unscale(double* __restrict__ d, int n, const unsigned* __r
 //   Bound: two grid barriers a round and the L2 traffic between them (A read by
 // halves and written, Q read and written: 66 MB a round at n = 1088).  The whole
 // eigensolve with this sweep in place of an FP64 one: n = 1088 86.8 -> 41.8 ms (60
-// -> 20 us a round), 1632 249 -> 126, 408 16.4 -> 14.0, 256 9.6 -> 8.3.  One barrier
+// -> 20 us a round), 1632 249 -> 126, 408 16.4 -> 14.0, 256 9.6 -> 8.3 (its products on
+// the tensor cores at the time).  One barrier
 // a round (the next round's rotations formed by the threads that make their
 // elements) gave 18 us there but was slower at 256 to 320; four rows of Q in flight
 // a thread changed nothing.

@@ -360,8 +360,8 @@ void local_kinetic(System& s, int nb, const double2* psi, int64_t ldp, double2* 
   constexpr bool kDf = std::is_same<T, df>::value;
   if constexpr (std::is_same<T, double>::value) {
     // the FP64 local part in double-float arithmetic on the FP32 pipes where
-    // the box has compiled passes (48-bit significands, relative rounding of
-    // about 2^-46 an operation)
+    // the box has compiled passes (48-bit significands, relative rounding of a
+    // sum below 2^-45)
     if (spec_box(s)) {
       local_kinetic<df>(s, nb, psi, ldp, hpsi, ldh, st, vnl, ldv);
       return;

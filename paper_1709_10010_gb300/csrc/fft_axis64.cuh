@@ -11,6 +11,8 @@
 // the radix-by-radix passes of the runtime plans), and no separate passes for the
 // pair densities and the Coulomb factor: exact exchange of 32 bands on 8 at 90^3 78.4
 // -> 57.9 ms.
+//   Boxes with another edge (50 among them: as 5 x 10 it has no coprime factors, and
+// no workload here has it) run the runtime plans.
 #pragma once
 #include "common.cuh"
 

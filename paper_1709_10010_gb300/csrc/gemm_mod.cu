@@ -13,15 +13,16 @@
 //   by more than 2^kPartGap gets an exponent for each, so that the smaller keeps its
 //   bits; the real products then are rebuilt one by one.  The only errors are
 //   the rounding to X (relative to |a| |b|: 2^-kT, 62 bits) and the final
-//   FP64 rounding: no product of slices is dropped, and the exponents follow
-//   the rows' norms, not their largest elements.
+//   FP64 rounding (the value within 2^-61, rounded once): no product of slices
+//   is dropped, and the exponents follow the rows' norms, not their largest
+//   elements.
 //
 // Work: 16 real BF16 products against the 36 of the integer-slice form (pairs
 // of base-128 digits) that this replaced, and one byte a modulus of partial
 // results instead of 36 FP32 partials per 4,096 of K.  Measured, a basis of
 // 1088 columns over 161,235 plane waves: A^H B with 544 columns and A B onto 544
-// columns together 29.4 ms, against 57.4 ms (12.9 and 17 ms; the residue GEMMs
-// 8.5 and 10.0 ms of them, tensor pipe 61-70% busy).
+// columns together 28.2 ms, against 57.4 ms (12.6 and 15.4 ms; tensor pipe of the
+// residue GEMMs 61-70% busy).
 //
 // Kernels: row and column norms; residues of the operands (BF16, K-major, one
 // plane a modulus); k_mod_gemm, one persistent pair of CTAs per two SMs; the
@@ -759,8 +760,9 @@ __device__ __forceinline__ void crt_store(const CrtOut& o, double re, double im,
 // two exponents); op(A) = A: (C[m][2n], C[m][2n+1]).  A block takes
 // 32 m (a warp's lanes: coalesced C) by NB n, its residues through shared
 // memory (16-byte loads, all in flight; pitch of an odd number of words), those of
-// several K ranges (RANGES) added modulo p on the way (20,000 x 544 outputs: 0.24 ms; 530
-// instructions an output, FP64 pipe 48% and issue slots 60% busy).
+// several K ranges (RANGES) added modulo p on the way.  Bound by its integer
+// instructions (1,088^2 outputs of A^H B 34 us, 5,000,000 x 1 of A B, mostly padding of
+// the 32 columns, 1.9 ms).
 template <bool CONJ, bool RANGES>
 __global__ void __launch_bounds__(256, 3)
     k_mod_crt(const unsigned char* __restrict__ res, int nz, int M, int N, int64_t Np,
