@@ -668,9 +668,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 // below 2^31; 64-bit multiply-adds on 31-bit digits ran at a quarter of their rate),
 // then carried into a 96-bit fraction.  Residues of several K ranges are added modulo
 // p first, and those of two products added as they are: a product that is zero has
-// residues that are all zero.  The fraction is off by at most 2^-95, 2^-94 of |a| |b|:
-// products of integers come out exact up to where |a| |b| passes 2^40 times the
-// result (2^24 with five digits).
+// residues that are all zero.  The fraction is off by at most 2^-95, which with P < 2^126
+// and integers of at least half 2^kT is 2^-91 of |a| |b|: products of integers come out
+// exact up to where |a| |b| passes 2^37 times the result (2^21 with five digits).
 struct CrtDigits {
   int d[kDigits] = {0, 0, 0, 0, 0, 0};
   template <int I> __device__ __forceinline__ void add(int r) {
@@ -687,6 +687,7 @@ struct CrtDigits {
 struct CrtFrac {
   unsigned long long h;  // leading 64 bits
   unsigned l;            // 32 more
+  unsigned exact;        // 1 when nothing was cut off below them
   __device__ __forceinline__ void set(const CrtDigits& c) {
     constexpr int M = (1 << 18) - 1;
     const int t4 = c.d[4] + (c.d[5] >> 18), t3 = c.d[3] + (t4 >> 18), t2 = c.d[2] + (t3 >> 18),
@@ -696,13 +697,15 @@ struct CrtFrac {
     const unsigned lo = (d1 << 28) | (d2 << 10) | (d3 >> 8);
     h = ((unsigned long long)hi << 32) | lo;
     l = (d3 << 24) | (d4 << 6) | (d5 >> 12);
+    exact = (d5 & 0xfff) == 0 ? 1u : 0u;
   }
   // the signed value times 2^(ea + eb - 2 kT), rounded once: the truncations
   // below add up to less than 2^-61 of it
   __device__ __forceinline__ double value(int ea, int eb) const {
     const bool neg = (long long)h < 0;
-    const unsigned lx = neg ? 0u - l : l;
-    const unsigned long long hx = neg ? ~h + (l == 0 ? 1ull : 0ull) : h;
+    // the magnitude cut off, so that opposite values have the same bits
+    const unsigned lx = neg ? ~l + exact : l;
+    const unsigned long long hx = neg ? ~h + (l == 0 ? exact : 0u) : h;
     if (hx == 0 && lx == 0) return 0.0;
     int s;
     unsigned long long w;
