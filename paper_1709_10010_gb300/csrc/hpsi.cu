@@ -17,26 +17,33 @@ namespace pwh {
 // threads take neighbouring elements of one band, whose 16-byte reads stay within
 // the band (scattered 16-byte writes filled half a sector each: the way out took
 // 1.40 ms for 512 bands of 161,235 plane waves and takes 0.46 as a gather).  One
-// range over all bands, so that few short bands fill their blocks (30^3, 2 to 12
-// bands: H 24.7 us, with a row of blocks a band 25.7 to 26.8).
-__global__ void __launch_bounds__(256) k_permute(const double2* __restrict__ src, int64_t lds, int64_t npw,
-                                                 int nb, const int32_t* __restrict__ idx,
+// range over all bands, so that few short bands fill their blocks (30^3, 4 bands: H
+// 24.8 us, with a row of blocks a band 26.9).  I: unsigned where that range has fewer
+// than 2^31 elements; a 64-bit division is most of a thread's work (80^3, 8 bands: H
+// 60.5 us with it, 57.6 without).
+template <typename I>
+__global__ void __launch_bounds__(256) k_permute(const double2* __restrict__ src, int64_t lds, I npw, I tot,
+                                                 const int32_t* __restrict__ idx,
                                                  double2* __restrict__ dst, int64_t ldd) {
-  const int64_t tot = npw * nb;
-  for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < tot; t += gridDim.x * (int64_t)256) {
-    const int64_t b = t / npw, i = t - b * npw;
-    dst[b * ldd + i] = src[b * lds + idx[i]];
+  for (I t = blockIdx.x * (I)256 + threadIdx.x; t < tot; t += gridDim.x * (I)256) {
+    const I b = t / npw, i = t - b * npw;
+    dst[(int64_t)b * ldd + i] = src[(int64_t)b * lds + idx[i]];
   }
 }
 
-static int permute_grid(int64_t npw, int nb) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>(152 * 16, (npw * nb + 255) / 256));
+static void permute(System& s, int nb, const double2* src, int64_t lds, const int32_t* idx, double2* dst,
+                    int64_t ldd) {
+  const int64_t tot = s.npw * (int64_t)nb;
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(152 * 16, (tot + 255) / 256));
+  if (tot < ((int64_t)1 << 31))
+    k_permute<unsigned><<<blocks, 256, 0, s.stream>>>(src, lds, (unsigned)s.npw, (unsigned)tot, idx, dst, ldd);
+  else
+    k_permute<int64_t><<<blocks, 256, 0, s.stream>>>(src, lds, s.npw, tot, idx, dst, ldd);
+  PWH_LAUNCH_CHECK();
 }
 
 void permute_public_to_internal(System& s, const double2* src, double2* dst, int nb, int64_t lds) {
-  k_permute<<<permute_grid(s.npw, nb), 256, 0, s.stream>>>(src, lds > 0 ? lds : s.npw, s.npw, nb,
-                                                          s.d_int_to_pub, dst, s.npw);
-  PWH_LAUNCH_CHECK();
+  permute(s, nb, src, lds > 0 ? lds : s.npw, s.d_int_to_pub, dst, s.npw);
 }
 
 void nonlocal_fp64(System& s, int nb, const double2* psi, int64_t ldp, double2* hpsi, int64_t ldh,
@@ -115,13 +122,9 @@ pwh_status pwh_apply_h(pwh_system* sys, int32_t nb, const void* psi, int64_t ld_
     ensure(s.ws_hpsi, n * sizeof(double2));
     double2* pi = (double2*)s.ws_psi.p;
     double2* hi = (double2*)s.ws_hpsi.p;
-    k_permute<<<permute_grid(s.npw, nb), 256, 0, s.stream>>>((const double2*)psi, ld_psi, s.npw, nb,
-                                                            s.d_int_to_pub, pi, s.npw);
-    PWH_LAUNCH_CHECK();
+    permute(s, nb, (const double2*)psi, ld_psi, s.d_int_to_pub, pi, s.npw);
     apply_internal(s, nb, pi, s.npw, hi, s.npw, s.precision);
-    k_permute<<<permute_grid(s.npw, nb), 256, 0, s.stream>>>(hi, s.npw, s.npw, nb, s.d_pub_to_int,
-                                                            (double2*)hpsi, ld_hpsi);
-    PWH_LAUNCH_CHECK();
+    permute(s, nb, hi, s.npw, s.d_pub_to_int, (double2*)hpsi, ld_hpsi);
   });
 }
 
