@@ -587,14 +587,16 @@ __global__ void __launch_bounds__(NT) ks_plane(cx<T>* __restrict__ W, int64_t wb
 template <typename T, int N>
 constexpr int plane_threads = std::is_same<T, float>::value ? (N >= 144 ? 1024 : N >= 120 ? 512 : 256)
                                                             : (N >= 96 ? 512 : 256);
-// FP32 where a launch has at most kFewPlanes blocks, about two an SM, so that a
-// block's own latency is the pass: 512 threads (one band, 256 / 512: 60 10.7 / 10.2 us,
-// 80 14.2 / 12.2, 90 15.7 / 13.8; four bands, 72 15.4 / 14.2, 90 28.6 / 26.0; below 48
-// no difference).
-constexpr int kFewPlanes = 360;
+// Where a launch has few blocks, so that a block's own latency is the pass.  FP32 up
+// to 360 blocks, about two an SM: 512 threads (one band, 256 / 512: 60 10.7 / 10.2 us, 80
+// 14.2 / 12.2, 90 15.7 / 13.8; four bands, 72 15.4 / 14.2, 90 28.6 / 26.0; below 48 no
+// difference).  Double-float up to one block an SM at 48 and 50 (H of one band, 256 /
+// 512: 48 65.7 / 63.9 us, 50 73.0 / 71.1; of four bands, more blocks than SMs, 65.7 / 101
+// and 77 / 117).
+template <typename T> constexpr int few_planes = std::is_same<T, float>::value ? 360 : 152;
 template <typename T, int N>
 constexpr int plane_threads_few =
-    std::is_same<T, float>::value && N >= 48 && N < 144 ? 512 : plane_threads<T, N>;
+    (std::is_same<T, float>::value ? N >= 48 && N < 144 : N >= 48 && N < 60) ? 512 : plane_threads<T, N>;
 template <int NT> using Threads = std::integral_constant<int, NT>;
 
 // Shared memory of the plane pass for `rows` rows per chunk.
@@ -752,7 +754,7 @@ template <typename T, int N> void spec_launch(SpecPass pass, System& s, const Pa
             W, a.wband, s.nsticks, s.ncols, s.d_stick_at, s.d_xcol, (const T*)a.V, s.plan[0].tw_off,
             tw, rows);
       };
-      if (N * a.bb <= kFewPlanes)
+      if (N * a.bb <= few_planes<T>)
         run(Threads<plane_threads_few<T, N>>{});
       else
         run(Threads<plane_threads<T, N>>{});

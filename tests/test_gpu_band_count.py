@@ -9,7 +9,7 @@ from paper_1709_10010_gb300 import synthetic as syn
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [30, 48, 60, 90, 96, 120])
+@pytest.mark.parametrize("n", [30, 48, 50, 60, 90, 96, 120])
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_band_alone_and_among_others(n, precision):
     import torch
